@@ -651,8 +651,8 @@ soc_status soc_nn_seed_features(const float *d_T, const float *d_T_prev, const f
  * {32, 64, ..., 256}; blocks_per_sm >= 1 (0 = occupancy maximum of the
  * default build; 4 or more selects the build limited to 64 registers per
  * thread, which keeps 4 blocks of 256 threads resident per SM); chunk in
- * [1, 1024] = packages per lane that a warp takes from the global work
- * counter at a time.
+ * [1, 1024] = most packages per lane that a warp takes from the global work
+ * counter at a time (fewer when little work is left).
  * Results do not depend on these settings.
  * ------------------------------------------------------------------------ */
 soc_status soc_set_launch(soc_ctx *ctx, int threads_per_block, int blocks_per_sm, int chunk);

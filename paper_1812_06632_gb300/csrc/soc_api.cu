@@ -873,9 +873,13 @@ static int32_t all_regular(const soc_ctx *ctx, const soc_batch_item *items, int 
     return 1;
 }
 
-// Launch shape of the tracer for `total` work indices.
-static void launch_geometry(soc_ctx *ctx, uint64_t total, bool regular, int &grid_out, int &variant)
+// Launch shape of the tracer for P.total work indices, and the share of the
+// remaining work a warp takes at a time (2^-take_shift, the power of two at
+// or below half a warp's even share).
+static void launch_geometry(soc_ctx *ctx, TraceParams &P, int &grid_out, int &variant)
 {
+    const uint64_t total = P.total;
+    const bool regular = P.regular != 0;
     variant = ctx->bps >= 4 ? 4 : 3;
     const int limit = std::max(1, ctx->occ[regular ? 1 : 0][variant - 3][ctx->tpb / 32 - 1]);
     const int per_sm = ctx->bps > 0 ? std::min(ctx->bps, limit) : limit;
@@ -884,6 +888,9 @@ static void launch_geometry(soc_ctx *ctx, uint64_t total, bool regular, int &gri
     const int64_t grid_need = (int64_t)((warps_needed * 32 + ctx->tpb - 1) / ctx->tpb);
     if (grid_need < grid) grid = grid_need < 1 ? 1 : grid_need;
     grid_out = (int)grid;
+    const uint64_t warps = (uint64_t)grid * (uint64_t)(ctx->tpb / 32);
+    P.take_shift = 1;
+    while (((uint64_t)1 << P.take_shift) < 2 * warps) ++P.take_shift;
 }
 
 // SOC_ERR_STATE when `s` is being captured into a CUDA graph: the direct
@@ -956,7 +963,7 @@ soc_status soc_simulate_frequency_batch_ex(soc_ctx *ctx, const soc_batch_item *i
         P.hot = one_cloud(ctx, items, n_items);
         P.regular = all_regular(ctx, items, n_items);
         int grid = 1, variant = 3;
-        launch_geometry(ctx, total, P.regular != 0, grid, variant);
+        launch_geometry(ctx, P, grid, variant);
         CK(launch_trace(P, grid, ctx->tpb, variant, s), "trace launch");
         // the host copies above used pageable buffers: they are staged before return
         return SOC_OK;
@@ -1030,7 +1037,7 @@ soc_status soc_batch_launch(soc_ctx *ctx, int batch_id, int64_t *d_tally, int64_
         P.hot = b.hot;
         P.regular = b.regular;
         int grid = 1, variant = 3;
-        launch_geometry(ctx, b.total, P.regular != 0, grid, variant);
+        launch_geometry(ctx, P, grid, variant);
         CK(launch_trace(P, grid, ctx->tpb, variant, s), "trace launch");
         return SOC_OK;
     });
@@ -1957,7 +1964,7 @@ extern "C" soc_status soc_simulate_frequency_batch_noalloc(soc_ctx *ctx, const s
         P.hot = one_cloud(ctx, items, n_items);
         P.regular = all_regular(ctx, items, n_items);
         int grid = 1, variant = 3;
-        launch_geometry(ctx, total, P.regular != 0, grid, variant);     // occupancy cached at soc_create
+        launch_geometry(ctx, P, grid, variant);     // occupancy cached at soc_create
         CK(launch_trace(P, grid, ctx->tpb, variant, s), "trace launch");
         return SOC_OK;
     });

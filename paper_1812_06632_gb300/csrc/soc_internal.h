@@ -65,6 +65,7 @@ struct TraceParams {
     int32_t n_items;
     uint32_t max_steps;
     int32_t chunk;
+    int32_t take_shift;          // a warp takes (work left) >> take_shift indices, within [32, 32 chunk]
     int32_t refill_min;          // refill a warp's idle lanes once this many are idle
     int32_t scatter_min;         // scatter a warp's waiting lanes once this many wait
     const int *abort_flag;       // host-mapped: nonzero = take no more work (soc_abort)
