@@ -507,6 +507,34 @@ __device__ __forceinline__ unsigned take_span(const TraceParams &P, unsigned lon
     return (unsigned)(want < 32u ? 32u : (want < most ? want : most));
 }
 
+// Adds the statistics of the lanes with `flush` to their items and clears
+// them (the whole warp calls it).  Lanes that share the first flushing lane's
+// item are summed first and make one set of atomics, since a set per lane
+// serialises at the item's 32-byte sector (155 000 lanes x 3 atomics at the
+// end of a launch alone); the other lanes, few and of several items, make
+// their own.
+__device__ __forceinline__ void flush_stats(unsigned long long *stats, unsigned long long (*acc)[256], int item, bool flush)
+{
+    const unsigned todo = __ballot_sync(kFull, flush);
+    if (todo == 0u) return;
+    const int it = __shfl_sync(kFull, item, __ffs(todo) - 1);
+    const bool mine = flush && item == it;
+#pragma unroll 1
+    for (int k = 0; k < 4; ++k) {
+        unsigned long long v = 0;
+        if (flush) { v = acc[k][threadIdx.x]; acc[k][threadIdx.x] = 0; }
+        // 27-bit pieces: 32 of them sum within 32 bits
+        const unsigned lo = __reduce_add_sync(kFull, mine ? (unsigned)v & 0x7FFFFFFu : 0u);
+        const unsigned mid = __reduce_add_sync(kFull, mine ? (unsigned)(v >> 27) & 0x7FFFFFFu : 0u);
+        const unsigned top = __reduce_add_sync(kFull, mine ? (unsigned)(v >> 54) : 0u);
+        if ((threadIdx.x & 31) == 0) {
+            const unsigned long long t = (unsigned long long)lo + ((unsigned long long)mid << 27) + ((unsigned long long)top << 54);
+            if (t) atomicAdd(stats + 4 * (long long)it + k, t);
+        }
+        if (flush && !mine && v) atomicAdd(stats + 4 * (long long)item + k, v);
+    }
+}
+
 template <int kMinBlocks, bool kSelf, bool kOneCloud, bool kRegular>
 __global__ void __launch_bounds__(256, kMinBlocks) trace_kernel(const TraceParams P)
 {
@@ -530,16 +558,13 @@ __global__ void __launch_bounds__(256, kMinBlocks) trace_kernel(const TraceParam
     uint64_t gidx = 0;
     // per-lane statistics, flushed when the lane moves to another item; the
     // sums live in shared memory (touched once per package) to spare registers
-    __shared__ unsigned long long s_acc[256][3];     // escaped, steps, emitted
-    unsigned long long *const acc = s_acc[threadIdx.x];
-    acc[0] = acc[1] = acc[2] = 0;
+    __shared__ unsigned long long s_acc[4][256];     // escaped, capped, steps, emitted
+    for (int k = 0; k < 4; ++k) s_acc[k][threadIdx.x] = 0;
     // octree launches: the lane's ancestors (regular-grid launches get no
     // dynamic shared memory and never touch them)
     extern __shared__ int32_t s_anc[];
     int32_t *const anc = s_anc + kAncRows * threadIdx.x;
     const DevCloud *C = P.clouds;             // the lane's cloud (used when !kOneCloud)
-    int acc_item = -1;
-    unsigned acc_cap = 0;
 
     for (;;) {
         unsigned idle = __ballot_sync(kFull, !active);
@@ -578,18 +603,28 @@ __global__ void __launch_bounds__(256, kMinBlocks) trace_kernel(const TraceParam
             const uint64_t avail = q_end - q_next;
             const int take = avail < (uint64_t)n_idle ? (int)avail : n_idle;
             const int rank = __popc(idle & lt_mask);
-            if (!active && rank < take) {
+            const bool get = !active && rank < take;
+            bool moved = false;              // the lane's packages come from another item now
+            int next_item = -1;
+            if (get) {
                 gidx = q_next + rank;
                 const int it_idx = find_item(P.prefix, P.n_items, gidx);
-                if (it_idx != item) {
-                    item = it_idx;
-                    const DevItem &IT = P.items[item];
+                moved = it_idx != item;
+                if (moved) {
+                    const DevItem &IT = P.items[it_idx];
                     C = P.clouds + IT.cloud;
                     const float2 kap = __ldg(C->kappa + IT.freq);
                     kabs = kap.x; ksca = kap.y;
                     g = __ldg(P.g_hg + IT.freq);
                     tally = P.tally + IT.tally_offset;
+                    next_item = it_idx;
                 }
+            }
+            if (__any_sync(kFull, moved)) {
+                flush_stats(P.stats, s_acc, item, moved && item >= 0);
+                if (moved) item = next_item;
+            }
+            if (get) {
                 const DevItem &IT = P.items[item];
                 const uint32_t pid = IT.pid_offset + (uint32_t)(gidx - P.prefix[item]);
                 r.init(P.seed, (uint32_t)IT.iteration, (uint32_t)IT.freq, pid, (uint32_t)IT.cloud,
@@ -600,18 +635,7 @@ __global__ void __launch_bounds__(256, kMinBlocks) trace_kernel(const TraceParam
                            ((kSelf && IT.source == SOC_SRC_DUST) ? kHomeBit : 0u);
                     set_inverse(p);
                     p.tauf = -log_pos(r.u());
-                    if (acc_item != item) {
-                        if (acc_item >= 0) {
-                            unsigned long long *st = P.stats + 4 * acc_item;
-                            if (acc[0]) atomicAdd(st + 0, acc[0]);
-                            if (acc_cap) atomicAdd(st + 1, (unsigned long long)acc_cap);
-                            if (acc[1]) atomicAdd(st + 2, acc[1]);
-                            if (acc[2]) atomicAdd(st + 3, acc[2]);
-                        }
-                        acc_item = item; acc_cap = 0;
-                        acc[0] = acc[1] = acc[2] = 0;
-                    }
-                    acc[2] += p.W;
+                    s_acc[3][threadIdx.x] += p.W;
                     active = true;
                 } else if (P.pkg_steps) {
                     P.pkg_steps[gidx] = 0;
@@ -675,21 +699,15 @@ __global__ void __launch_bounds__(256, kMinBlocks) trace_kernel(const TraceParam
                         atomicAdd(P.self + (tally - P.tally) + p.cell, (unsigned long long)p.pend);
                 }
                 p.pend = 0;
-                if (res == kEscaped) acc[0] += p.W;
-                if (res == kCapped) acc_cap += 1;
-                acc[1] += p.steps;
+                if (res == kEscaped) s_acc[0][threadIdx.x] += p.W;
+                if (res == kCapped) s_acc[1][threadIdx.x] += 1;
+                s_acc[2][threadIdx.x] += p.steps;
                 if (P.pkg_steps) P.pkg_steps[gidx] = p.steps;
                 active = false;
             }
         }
     }
-    if (acc_item >= 0) {
-        unsigned long long *st = P.stats + 4 * acc_item;
-        if (acc[0]) atomicAdd(st + 0, acc[0]);
-        if (acc_cap) atomicAdd(st + 1, (unsigned long long)acc_cap);
-        if (acc[1]) atomicAdd(st + 2, acc[1]);
-        if (acc[2]) atomicAdd(st + 3, acc[2]);
-    }
+    flush_stats(P.stats, s_acc, item, item >= 0);
 }
 
 // ---------------------------------------------------------------------------
