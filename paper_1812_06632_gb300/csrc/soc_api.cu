@@ -701,7 +701,7 @@ soc_status soc_dust_upload(soc_ctx *ctx, int n_freq, const double *nu, const dou
         CK(ctx->d_kabs.alloc(n_freq), "alloc");
         CK(ctx->d_lnE.alloc(kTableN), "alloc");
         CK(ctx->d_lnT.alloc(kTableN), "alloc");
-        CK(ctx->d_lmax.alloc(n_freq), "alloc");
+        CK(ctx->d_lmax.alloc(2 * (size_t)n_freq), "alloc");     // see launch_dust_emission
         CK(cudaMemcpy(ctx->d_g.p, gf.data(), 4 * n_freq, cudaMemcpyHostToDevice), "copy");
         CK(cudaMemcpy(ctx->d_w.p, ctx->w.data(), 8 * n_freq, cudaMemcpyHostToDevice), "copy");
         CK(cudaMemcpy(ctx->d_w_kabs.p, wk.data(), 8 * n_freq, cudaMemcpyHostToDevice), "copy");

@@ -197,48 +197,392 @@ __device__ __forceinline__ double dust_L(const DevCloud &C, const TempTables &tt
     return __dmul_rn(__dmul_rn(__dmul_rn(__dmul_rn(4.0 * kPi, rho), V), __ldg(tt.kabs + f)), B);
 }
 
-// Luminosities of every (frequency, leaf) and their maximum per frequency.
-// L is kept in the weight array (FP64 bits in the uint64 slots) for
-// dust_weight_kernel, which turns it into the weight in place: one Planck
-// evaluation per (leaf, frequency) instead of two.
-__global__ void dust_max_kernel(const DevCloud *__restrict__ dcl, int64_t n_leaf, const TempTables tt,
-                                const float *__restrict__ T, int freq_lo, int n_freq,
-                                unsigned long long *Lmax, double *__restrict__ Lout)
+// ---------------------------------------------------------------------------
+// Uniform dust weights: W = rint(RN(RN(L / m) 2^31)) for every (frequency,
+// leaf), m = max over the leaves of L at that frequency, L in FP64 (dust_L).
+//
+// Evaluating L in FP64 costs about 50 FP64 operations (expm1 and three
+// divisions) on a pipe that issues 2 lanes per clock and SM: 13.4 ms for the
+// maxima and 3.1 ms for the weights of 2.1e6 leaves x 64 frequencies, where
+// the 1.07 GB of weights written take 0.16 ms.  The results are a maximum and
+// a rounded integer, so almost every value is settled by a cheaper bound:
+//   dust_bound_kernel  maxima of l ~ log2 L from FP32 (2 MUFU operations);
+//   dust_max_kernel    the same l again: only leaves within kMaxSlack of
+//                      their frequency's maximum (or whose l is not reliable)
+//                      have L evaluated in FP64 and compared, so m is the
+//                      FP64 maximum itself;
+//   dust_weight_kernel v = L / m 2^31 from pairs of FP32 numbers (hi + lo,
+//                      about 2^-42 relative) with an error bound; where the
+//                      bound leaves the rounding open, or an operand is
+//                      outside the ranges the bound covers, W is evaluated
+//                      in FP64 as above.
+// m, the weights and e_unit are therefore the FP64 evaluation's, bit for bit.
+// Measured on the same leaves: 0.13, 0.22 and 1.1 ms.
+// A thread takes leaves, a block kDustF frequencies (blockIdx.y) whose
+// constants it prepares in shared memory.
+// ---------------------------------------------------------------------------
+constexpr int kDustF = 16;               // frequencies per block
+constexpr int kDustLeaves = 4;           // leaves a thread holds in the bound and maximum passes
+constexpr float kMaxSlack = 0x1p-8f;     // twice the error of l (< 1.6e-3) and a margin
+constexpr float kInf = __builtin_huge_valf();
+
+struct DustFreq {
+    float ch, cl;                        // log2(e) h nu / k (K), hi + lo
+    float lf, lpre;                      // log2(kabs pre), log2(pre), pre = 2 h nu^3 / c^2; lpre = -inf: no bound
+    float sh, sl;                        // mantissa of kabs pre 2^31 / m, hi + lo (weights only)
+    int32_t se;                          // its exponent; kSeZero: m = 0, kSeSlow: no bound
+    int32_t pad;
+};
+constexpr int32_t kSeZero = 1 << 20, kSeSlow = 1 << 21;
+
+__device__ __forceinline__ float lg2(float v) { float r; asm("lg2.approx.f32 %0, %1;" : "=f"(r) : "f"(v)); return r; }
+__device__ __forceinline__ float ex2(float v) { float r; asm("ex2.approx.f32 %0, %1;" : "=f"(r) : "f"(v)); return r; }
+__device__ __forceinline__ float rcp(float v) { float r; asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(v)); return r; }
+
+__device__ __forceinline__ int exponent_of(double v) { return (int)((__double_as_longlong(v) >> 52) & 0x7FF) - 1023; }
+__device__ __forceinline__ double mantissa_of(double v)
 {
-    const DevCloud &C = *dcl;
-    for (int fi = 0; fi < n_freq; ++fi) {
-        double m = 0.0;
-        for (int64_t li = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; li < n_leaf;
-             li += (int64_t)gridDim.x * blockDim.x) {
-            const double L = dust_L(C, tt, T, __ldg(C.leaf + li), freq_lo + fi);
-            Lout[(int64_t)fi * n_leaf + li] = L;
-            m = L > m ? L : m;
+    return __longlong_as_double((__double_as_longlong(v) & 0x000FFFFFFFFFFFFFll) | 0x3FF0000000000000ll);
+}
+
+// Constants of frequency f (one thread each; m only for the weights).
+__device__ __forceinline__ DustFreq dust_freq(const TempTables &tt, int f, double m, bool weights)
+{
+    DustFreq d;
+    const double nu = __ldg(tt.nu + f), kabs = __ldg(tt.kabs + f);
+    const double c = 1.4426950408889634 * (kH * nu / kK);
+    const double pre = 2.0 * kH * (nu * nu * nu) / (kC * kC);
+    const double kp = kabs * pre;
+    d.ch = (float)c;
+    d.cl = (float)(c - (double)d.ch);
+    const bool ok = pre > 0x1p-100 && pre < 0x1p300 && kabs > 0x1p-200 && kabs < 0x1p200 && c > 0x1p-60 && c < 0x1p60;
+    d.lf = ok ? (float)exponent_of(kp) + lg2((float)mantissa_of(kp)) : 0.f;
+    d.lpre = ok ? (float)exponent_of(pre) + lg2((float)mantissa_of(pre)) : -kInf;
+    d.sh = d.sl = 0.f;
+    d.se = 0;
+    if (weights) {
+        if (m == 0.0) {
+            d.se = kSeZero;
+        } else if (!ok || !(m > 0x1p-600 && m < 0x1p600)) {
+            d.se = kSeSlow;
+        } else {
+            const double s = kp / m, sm = mantissa_of(s);
+            d.se = exponent_of(s) + 31;
+            d.sh = (float)sm;
+            d.sl = (float)(sm - (double)d.sh);
         }
-        block_max_to(m, Lmax + fi);
-        __syncthreads();
+    }
+    return d;
+}
+
+// A leaf's side of the bound: 1/T and log2(4 pi rho V) in FP32.  zero: rho = 0
+// (L = 0); ok: T, rho and V inside the ranges the bound covers.
+struct DustLeaf {
+    float it, lg;
+    bool ok, zero;
+};
+
+__device__ __forceinline__ bool dust_ranges(float T, float rho, double V)
+{
+    // V > 0 in [2^-200, 2^300) by its exponent bits: no FP64 comparison
+    const unsigned e = (unsigned)((unsigned long long)__double_as_longlong(V) >> 52);
+    return T > 1e-3f && T < 1e6f && (rho == 0.0f || (rho > 0x1p-100f && rho < 0x1p100f)) && e - 823u < 500u;
+}
+
+__device__ __forceinline__ DustLeaf dust_leaf(float T, float rho, double V)
+{
+    DustLeaf d;
+    d.ok = dust_ranges(T, rho, V);
+    d.zero = rho == 0.0f;
+    d.it = __frcp_rn(T);
+    const uint64_t b = (uint64_t)__double_as_longlong(V);
+    const float vm = __uint_as_float(0x3f800000u | (uint32_t)((b >> 29) & 0x7FFFFFu));
+    d.lg = __fadd_rn(__fadd_rn((float)((int)(b >> 52) - 1023), lg2(vm)), __fadd_rn(3.6514961f, lg2(rho)));   // log2(4 pi)
+    return d;
+}
+
+// l ~ log2 L, within 1e-3 + 2e-6 / y for y = log2(e) h nu / (k T) in [2^-8,
+// 1024]; reliable: that range, and L (and the Planck function) a normal
+// FP64 number, so that its FP64 evaluation has its full precision.
+__device__ __forceinline__ float dust_log2(const DustFreq &f, const DustLeaf &c, float &y, bool &reliable)
+{
+    y = __fmul_rn(f.ch, c.it);
+    const float l = __fsub_rn(__fsub_rn(__fadd_rn(c.lg, f.lf), y), lg2(__fsub_rn(1.0f, ex2(-y))));
+    reliable = c.ok && y >= 0x1p-8f && __fsub_rn(f.lpre, y) > -1015.0f && l > -1015.0f && l < 1015.0f;
+    return l;
+}
+
+__device__ __forceinline__ uint32_t ordered(float v)      // increasing in v; 0 is below every float
+{
+    const uint32_t b = __float_as_uint(v);
+    return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
+}
+
+__device__ __forceinline__ float unordered(uint32_t u)    // inverse of ordered; 0 -> -inf
+{
+    if (u == 0u) return -kInf;
+    return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
+}
+
+__device__ __forceinline__ void load_dust_freqs(DustFreq *s_f, const TempTables &tt, int freq_lo, int f0, int nf,
+                                                const unsigned long long *Lmax)
+{
+    if ((int)threadIdx.x < nf)
+        s_f[threadIdx.x] = dust_freq(tt, freq_lo + f0 + threadIdx.x,
+                                     Lmax ? __longlong_as_double((long long)Lmax[f0 + threadIdx.x]) : 0.0, Lmax != nullptr);
+    __syncthreads();
+}
+
+// lmax[f] (ordered) = max of the reliable l of frequency f.
+__global__ void __launch_bounds__(256) dust_bound_kernel(const DevCloud *__restrict__ dcl, int64_t n_leaf,
+                                                         const TempTables tt, const float *__restrict__ T, int freq_lo,
+                                                         int n_freq, unsigned *lmax)
+{
+    __shared__ DustFreq s_f[kDustF];
+    __shared__ uint32_t s_max[8][kDustF];
+    const int f0 = blockIdx.y * kDustF, nf = min(kDustF, n_freq - f0);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    load_dust_freqs(s_f, tt, freq_lo, f0, nf, nullptr);
+    const DevCloud &C = *dcl;
+    uint32_t run = 0;                     // lane f: this warp's maximum of frequency f0 + f
+    const int64_t tile = 256 * kDustLeaves;
+    for (int64_t b = blockIdx.x * tile; b < n_leaf; b += gridDim.x * tile) {
+        DustLeaf c[kDustLeaves];
+#pragma unroll
+        for (int k = 0; k < kDustLeaves; ++k) {
+            const int64_t li = b + k * 256 + threadIdx.x;
+            c[k].ok = false;
+            if (li < n_leaf) {
+                const int32_t cell = __ldg(C.leaf + li);
+                c[k] = dust_leaf(__ldg(T + cell), __ldg(C.rho + cell), __ldg(C.volume + cell));
+                if (c[k].zero) c[k].ok = false;
+            }
+        }
+        for (int f = 0; f < nf; ++f) {
+            uint32_t m = 0;
+#pragma unroll
+            for (int k = 0; k < kDustLeaves; ++k) {
+                float y;
+                bool rel;
+                const float l = dust_log2(s_f[f], c[k], y, rel);
+                if (rel) m = max(m, ordered(l));
+            }
+            m = __reduce_max_sync(0xffffffffu, m);
+            if (lane == f) run = max(run, m);
+        }
+    }
+    if (lane < kDustF) s_max[warp][lane] = run;
+    __syncthreads();
+    if ((int)threadIdx.x < nf) {
+        uint32_t m = 0;
+        for (int w = 0; w < 8; ++w) m = max(m, s_max[w][threadIdx.x]);
+        if (m) atomicMax(lmax + f0 + threadIdx.x, m);
     }
 }
 
-__global__ void dust_weight_kernel(const DevCloud *__restrict__ dcl, int64_t n_leaf, const TempTables tt,
-                                   const float *__restrict__ T, int freq_lo, int n_freq, uint32_t n_per_cell,
-                                   const unsigned long long *__restrict__ Lmax, unsigned long long *w,
-                                   double *e_unit)
+// FP64 luminosity of a leaf compared with the running maximum (rare: kept out
+// of line so that it does not raise the callers' register count).
+__device__ __noinline__ void dust_max_exact(const DevCloud &C, const TempTables &tt, const float *T, int32_t cell, int f,
+                                            unsigned long long *out)
 {
-    const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (tid < n_freq) {
-        const double m = __longlong_as_double((long long)Lmax[tid]);
-        e_unit[tid] = __ddiv_rn(__ddiv_rn(m, (double)n_per_cell), kWUnit);
-    }
-    for (int64_t li = tid; li < n_leaf; li += (int64_t)gridDim.x * blockDim.x) {
-        for (int fi = 0; fi < n_freq; ++fi) {
-            const double m = __longlong_as_double((long long)__ldg(Lmax + fi));
-            unsigned long long &slot = w[(int64_t)fi * n_leaf + li];
-            unsigned long long W = 0;
-            if (m > 0.0) {
-                const double L = __longlong_as_double((long long)slot);   // from dust_max_kernel
-                W = (unsigned long long)rint(__dmul_rn(__ddiv_rn(L, m), kWUnit));
+    const double L = dust_L(C, tt, T, cell, f);
+    if (!(L > 0.0)) return;
+    const unsigned long long b = (unsigned long long)__double_as_longlong(L);
+    // equal maxima (leaves of one temperature and density) skip the atomic
+    if (b > *reinterpret_cast<volatile unsigned long long *>(out)) atomicMax(out, b);
+}
+
+// Lmax[f] = max of L over the leaves, as FP64 bits.
+__global__ void __launch_bounds__(256) dust_max_kernel(const DevCloud *__restrict__ dcl, int64_t n_leaf,
+                                                       const TempTables tt, const float *__restrict__ T, int freq_lo,
+                                                       int n_freq, const unsigned *__restrict__ lmax,
+                                                       unsigned long long *Lmax)
+{
+    __shared__ DustFreq s_f[kDustF];
+    __shared__ float s_thr[kDustF];
+    const int f0 = blockIdx.y * kDustF, nf = min(kDustF, n_freq - f0);
+    if ((int)threadIdx.x < nf) s_thr[threadIdx.x] = __fsub_rn(unordered(__ldg(lmax + f0 + threadIdx.x)), kMaxSlack);
+    load_dust_freqs(s_f, tt, freq_lo, f0, nf, nullptr);
+    const DevCloud &C = *dcl;
+    const int64_t tile = 256 * kDustLeaves;
+    for (int64_t b = blockIdx.x * tile; b < n_leaf; b += gridDim.x * tile) {
+        DustLeaf c[kDustLeaves];
+        int32_t cell[kDustLeaves];
+#pragma unroll
+        for (int k = 0; k < kDustLeaves; ++k) {
+            const int64_t li = b + k * 256 + threadIdx.x;
+            c[k] = DustLeaf{1.0f, 0.0f, true, true};
+            cell[k] = 0;
+            if (li < n_leaf) {
+                cell[k] = __ldg(C.leaf + li);
+                c[k] = dust_leaf(__ldg(T + cell[k]), __ldg(C.rho + cell[k]), __ldg(C.volume + cell[k]));
             }
-            slot = W;
+        }
+        for (int f = 0; f < nf; ++f) {
+#pragma unroll
+            for (int k = 0; k < kDustLeaves; ++k) {
+                float y;
+                bool rel;
+                const float l = dust_log2(s_f[f], c[k], y, rel);
+                // certainly below the maximum: no density, L = 0 because
+                // expm1 overflows (y > 1024), or l below the limit, by 2^64
+                // where the FP64 evaluation may be a subnormal's (which is at
+                // most 2^12 above the value)
+                const bool nil = c[k].ok && (c[k].zero || (s_f[f].lpre > -kInf && y >= 0x1p-8f &&
+                                                           (y > 1030.0f || l < (rel ? s_thr[f] : s_thr[f] - 64.0f))));
+                if (!nil) dust_max_exact(C, tt, T, cell[k], freq_lo + f0 + f, Lmax + f0 + f);
+            }
+        }
+    }
+}
+
+// 2^(j/32) - 1 as hi + lo, j = 0 .. 31 (Taylor series of exp(j ln2 / 32)).
+struct Exp2Table { float h[32], l[32]; };
+constexpr Exp2Table make_exp2_table()
+{
+    Exp2Table t{};
+    for (int j = 0; j < 32; ++j) {
+        const double a = 0.69314718055994530942 * j / 32.0;
+        double term = 1.0, sum = 0.0;
+        for (int n = 1; n < 24; ++n) { term = term * a / n; sum += term; }
+        t.h[j] = (float)sum;
+        t.l[j] = (float)(sum - (double)t.h[j]);
+    }
+    return t;
+}
+__device__ const Exp2Table g_exp2_table = make_exp2_table();
+
+__device__ __noinline__ unsigned long long dust_weight_exact(const DevCloud &C, const TempTables &tt, const float *T,
+                                                             int32_t cell, int f, double m)
+{
+    const double L = dust_L(C, tt, T, cell, f);
+    return (unsigned long long)rint(__dmul_rn(__ddiv_rn(L, m), kWUnit));
+}
+
+// A sum of FP32 numbers a + b = s + e exactly (Knuth's two-sum; the short
+// form needs |a| >= |b| or a = 0).
+__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
+{
+    s = __fadd_rn(a, b);
+    const float t = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+}
+__device__ __forceinline__ void quick_two_sum(float a, float b, float &s, float &e)
+{
+    const float t = __fadd_rn(a, b);
+    e = __fsub_rn(b, __fsub_rn(t, a));
+    s = t;
+}
+
+__global__ void __launch_bounds__(256) dust_weight_kernel(const DevCloud *__restrict__ dcl, int64_t n_leaf,
+                                                          const TempTables tt, const float *__restrict__ T, int freq_lo,
+                                                          int n_freq, uint32_t n_per_cell,
+                                                          const unsigned long long *__restrict__ Lmax,
+                                                          unsigned long long *w, double *e_unit)
+{
+    __shared__ DustFreq s_f[kDustF];
+    const int f0 = blockIdx.y * kDustF, nf = min(kDustF, n_freq - f0);
+    const int lane = threadIdx.x & 31;
+    const float th = g_exp2_table.h[lane], tl = g_exp2_table.l[lane];
+    load_dust_freqs(s_f, tt, freq_lo, f0, nf, Lmax);
+    if (blockIdx.x == 0 && (int)threadIdx.x < nf) {
+        const double m = __longlong_as_double((long long)Lmax[f0 + threadIdx.x]);
+        e_unit[f0 + threadIdx.x] = __ddiv_rn(__ddiv_rn(m, (double)n_per_cell), kWUnit);
+    }
+    const DevCloud &C = *dcl;
+    constexpr float kLn2H = 0x1.62e43p-1f, kLn2L = -0x1.05c61p-29f;          // ln 2, hi + lo
+    constexpr float k4PiH = 0x1.921fb6p+3f, k4PiL = -0x1.777a5cp-22f;        // 4 pi, hi + lo
+    for (int64_t b = blockIdx.x * (int64_t)256; b < n_leaf; b += (int64_t)gridDim.x * 256) {
+        const int64_t li = b + threadIdx.x;
+        const bool in = li < n_leaf;                 // every lane of the warp takes part in the shuffles
+        const int32_t cell = in ? __ldg(C.leaf + li) : 0;
+        const float t = in ? __ldg(T + cell) : 1.0f, rho = in ? __ldg(C.rho + cell) : 0.0f;
+        const double V = in ? __ldg(C.volume + cell) : 1.0;
+        const bool ok = dust_ranges(t, rho, V);
+        // 1/T and the mantissa of 4 pi rho V as hi + lo, its exponent ge
+        const float ih = __frcp_rn(t), il = __fmul_rn(__fmaf_rn(-t, ih, 1.0f), ih);
+        const uint64_t vb = (uint64_t)__double_as_longlong(V);
+        const float vh = __uint_as_float(0x3f800000u | (uint32_t)((vb >> 29) & 0x7FFFFFu));
+        const float vl = __fmul_rn(__uint2float_rn((uint32_t)(vb & 0x1FFFFFFFu)), 0x1p-52f);
+        const uint32_t rb = __float_as_uint(rho);
+        const float rm = __uint_as_float(0x3f800000u | (rb & 0x7FFFFFu));
+        const int ge = (int)(vb >> 52) - 1023 + (int)(rb >> 23) - 127;
+        const float r4h = __fmul_rn(rm, k4PiH), r4l = __fmaf_rn(rm, k4PiL, __fmaf_rn(rm, k4PiH, -r4h));
+        const float gh = __fmul_rn(r4h, vh);
+        const float gl = __fmaf_rn(r4l, vh, __fmaf_rn(r4h, vl, __fmaf_rn(r4h, vh, -gh)));
+        for (int f = 0; f < nf; ++f) {
+            const DustFreq F = s_f[f];
+            // y = log2(e) h nu / (k T) = n / 32 + s, |s| <= 1/64
+            const float p = __fmul_rn(F.ch, ih);
+            const float pe = __fmaf_rn(F.cl, ih, __fmaf_rn(F.ch, il, __fmaf_rn(F.ch, ih, -p)));
+            const float tn = __fmaf_rn(fminf(p, 2048.0f), 32.0f, 12582912.0f);
+            const int n = __float_as_int(tn) - 0x4B400000;
+            const int k = n >> 5, e = ge + F.se - k;
+            // W = 0: no density, an overflowing expm1 (y > 1024), a maximum
+            // of 0, or v < 1/2 (the mantissas' quotient is below
+            // 4 / (2^2^-8 - 1) < 2^11); whole warps of such leaves are
+            // common where the maximum is a hot leaf's
+            const bool plain = ok && F.se < kSeZero && p >= 0x1p-8f;
+            const bool zero = !in || F.se == kSeZero || (plain && (rho == 0.0f || p > 1030.0f || e < -16));
+            if (__all_sync(0xffffffffu, zero)) {
+                if (in) w[(int64_t)(f0 + f) * n_leaf + li] = 0;
+                continue;
+            }
+            const float d = __fmaf_rn(__fsub_rn(tn, 12582912.0f), -0.03125f, p);
+            float sh, sl;
+            two_sum(d, pe, sh, sl);
+            // a = e^(s ln2) - 1 (Taylor to the fifth power)
+            const float rh = __fmul_rn(sh, kLn2H);
+            const float rl = __fmaf_rn(sl, kLn2H, __fmaf_rn(sh, kLn2L, __fmaf_rn(sh, kLn2H, -rh)));
+            const float r2 = __fmul_rn(rh, rh);
+            const float r2l = __fmaf_rn(__fadd_rn(rh, rh), rl, __fmaf_rn(rh, rh, -r2));
+            const float q = __fmul_rn(__fmul_rn(rh, r2), __fmaf_rn(rh, __fmaf_rn(rh, 0x1.111112p-7f, 0x1.555556p-5f),
+                                                                   0x1.555556p-3f));
+            float ah, al;
+            quick_two_sum(rh, __fmul_rn(0.5f, r2), ah, al);
+            al = __fadd_rn(al, __fadd_rn(__fmaf_rn(0.5f, r2l, rl), q));
+            // 2^(n/32 - k) e^(s ln2) - 1 = t + a + t a, t = 2^(j/32) - 1
+            const float t1 = __shfl_sync(0xffffffffu, th, n & 31), t1l = __shfl_sync(0xffffffffu, tl, n & 31);
+            const float ta = __fmul_rn(t1, ah);
+            const float tal = __fmaf_rn(t1l, ah, __fmaf_rn(t1, al, __fmaf_rn(t1, ah, -ta)));
+            float s1, e1, s2, e2;
+            quick_two_sum(t1, ah, s1, e1);
+            quick_two_sum(s1, ta, s2, e2);
+            const float lo = __fadd_rn(__fadd_rn(__fadd_rn(e1, e2), __fadd_rn(al, tal)), t1l);
+            // (e^x - 1) 2^-k = (1 - 2^-k) + that
+            const float mk = k < 120 ? __uint_as_float((uint32_t)(127 - max(k, 0)) << 23) : 0.0f;
+            const float c1 = __fsub_rn(1.0f, mk), ce = __fsub_rn(__fsub_rn(1.0f, c1), mk);
+            float eh, el;
+            two_sum(c1, s2, eh, el);
+            // normalised: the quotient's correction is good to (el / eh)^2
+            quick_two_sum(eh, __fadd_rn(el, __fadd_rn(ce, lo)), eh, el);
+            // v = g s / (e^x - 1)
+            const float nh = __fmul_rn(gh, F.sh);
+            const float nl = __fmaf_rn(gl, F.sh, __fmaf_rn(gh, F.sl, __fmaf_rn(gh, F.sh, -nh)));
+            const float rc = rcp(eh);
+            const float qh = __fmul_rn(nh, rc);
+            const float ql = __fmul_rn(__fmaf_rn(-qh, el, __fadd_rn(__fmaf_rn(-qh, eh, nh), nl)), rc);
+            unsigned long long W = 0;
+            bool open = !zero && (!plain || e > 40);
+            if (!zero && !open) {
+                const float sc = __uint_as_float((uint32_t)(127 + e) << 23);
+                const float vvh = __fmul_rn(qh, sc), vvl = __fmul_rn(ql, sc);
+                if (vvh >= 0.49f) {
+                    const uint32_t ni = __float2uint_rn(vvh);
+                    const float rem = __fadd_rn(__fsub_rn(vvh, __uint2float_rn(ni)), vvl);
+                    const float dr = rintf(rem);
+                    // bound on the error of v: of the pairs above, 1 / (e^x
+                    // - 1) where 2^-k (e^x - 1) is small, the exponent y and
+                    // the FP32 remainder (errors of at most 0.4 of it against
+                    // extended precision over x = 0.005 .. 600)
+                    const float err = __fmaf_rn(vvh, __fmaf_rn(p, 0x1p-44f, __fmaf_rn(rc, 0x1p-42f, 0x1p-42f)), 0x1p-20f);
+                    W = ni + (uint32_t)__float2int_rn(dr);      // 32 bits: a 64-bit conversion is an FP64 operation
+                    open = !(fabsf(__fsub_rn(rem, dr)) < __fsub_rn(0.5f, err)) || !(vvh < 2148000000.0f) || p > 900.0f;
+                }
+            }
+            if (open)
+                W = dust_weight_exact(C, tt, T, cell, freq_lo + f0 + f, __longlong_as_double((long long)__ldg(Lmax + f0 + f)));
+            if (in) w[(int64_t)(f0 + f) * n_leaf + li] = W;
         }
     }
 }
@@ -656,15 +1000,21 @@ cudaError_t launch_dust_emission(const DevCloud *dcl, int64_t n_leaf, const Temp
                                  int freq_lo, int n_freq, uint32_t n_per_cell, uint64_t *w, double *e_unit,
                                  unsigned long long *scratch_max, cudaStream_t s)
 {
-    cudaError_t e = cudaMemsetAsync(scratch_max, 0, sizeof(unsigned long long) * n_freq, s);
+    // scratch: [n_freq] maxima of L (FP64 bits), then [n_freq] maxima of its bound
+    cudaError_t e = cudaMemsetAsync(scratch_max, 0, 2 * sizeof(unsigned long long) * n_freq, s);
     if (e != cudaSuccess) return e;
-    dust_max_kernel<<<grid_for(n_leaf, 256), 256, 0, s>>>(dcl, n_leaf, tt, T, freq_lo, n_freq, scratch_max,
-                                                          reinterpret_cast<double *>(w));
+    unsigned *lmax = reinterpret_cast<unsigned *>(scratch_max + n_freq);
+    const unsigned fy = (unsigned)((n_freq + kDustF - 1) / kDustF);
+    const unsigned cap = std::max(1u, (unsigned)(grid_for((int64_t)1 << 40, 256) / fy));      // about 8 blocks per SM in all
+    const int64_t tile = 256 * kDustLeaves;
+    const dim3 g1((unsigned)std::min<int64_t>((n_leaf + tile - 1) / tile, cap), fy);
+    const dim3 g2((unsigned)std::min<int64_t>((n_leaf + 255) / 256, cap), fy);
+    dust_bound_kernel<<<g1, 256, 0, s>>>(dcl, n_leaf, tt, T, freq_lo, n_freq, lmax);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const int64_t n = n_leaf > n_freq ? n_leaf : n_freq;
-    dust_weight_kernel<<<grid_for(n, 256), 256, 0, s>>>(dcl, n_leaf, tt, T, freq_lo, n_freq, n_per_cell,
-                                                         scratch_max, reinterpret_cast<unsigned long long *>(w),
-                                                         e_unit);
+    dust_max_kernel<<<g1, 256, 0, s>>>(dcl, n_leaf, tt, T, freq_lo, n_freq, lmax, scratch_max);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    dust_weight_kernel<<<g2, 256, 0, s>>>(dcl, n_leaf, tt, T, freq_lo, n_freq, n_per_cell, scratch_max,
+                                          reinterpret_cast<unsigned long long *>(w), e_unit);
     return cudaGetLastError();
 }
 
