@@ -34,11 +34,33 @@ __device__ __forceinline__ double planck(double nu, double T)
 // cell; kShared, dynamic shared memory for n_freq doubles) or per cell (very
 // long frequency tables), the sum over frequencies per cell in frequency
 // order either way.
+//
+// The FP64 pipe (2 lanes a clock and SM) bounds this kernel.  A conversion, a
+// multiplication and an addition per counter took 0.82 ms for 2.1e6 cells x
+// 64 frequencies (1.07 GB, 0.16 ms at the copy rate).  Counters below 2^52
+// need no conversion: v placed in the mantissa of 2^52 is the number 2^52 + v,
+// and fma(w, 2^52 + v, -w 2^52) is the product w v with its one rounding.
+// Four counters are loaded before their sum so that the loads overlap, and one
+// test of the four takes them all to the short product (a test per counter
+// made both forms execute: 1.05 ms).  0.54 ms.
 constexpr int kWfShared = 4096;
 
 __device__ __forceinline__ double wf_of(const double *s_wf, const double *w, const double *e_unit, int f, bool shared)
 {
     return shared ? s_wf[f] : __dmul_rn(__ldg(w + f), __ldg(e_unit + f));
+}
+
+// RN(w v), v in [0, 2^52) and w of normal magnitude (see plain_weight).
+__device__ __forceinline__ double weighted_count(double w, long long v)
+{
+    // -w 2^52, formed on the exponent bits
+    return __fma_rn(w, __longlong_as_double(v | 0x4330000000000000ll),
+                    __longlong_as_double((__double_as_longlong(w) + (52ll << 52)) ^ (1ll << 63)));
+}
+
+__device__ __forceinline__ bool plain_weight(double w)
+{
+    return (((unsigned)(__double_as_longlong(w) >> 52) & 0x7FFu) - 124u) < 1700u;
 }
 
 template <bool kShared>
@@ -48,9 +70,13 @@ __global__ void absorbed_power_kernel(const DevCloud *__restrict__ dcl, int64_t 
                                       int n_freq, const double *A_in, double *A_out)
 {
     extern __shared__ double s_wf[];
+    bool plain = kShared;                // every weight takes the short product
     if (kShared) {
-        for (int f = threadIdx.x; f < n_freq; f += blockDim.x) s_wf[f] = __dmul_rn(__ldg(w + f), __ldg(e_unit + f));
-        __syncthreads();
+        for (int f = threadIdx.x; f < n_freq; f += blockDim.x) {
+            s_wf[f] = __dmul_rn(__ldg(w + f), __ldg(e_unit + f));
+            plain = plain && plain_weight(s_wf[f]);
+        }
+        plain = __syncthreads_and(plain);
     }
     const DevCloud &C = *dcl;
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < n_cells;
@@ -59,9 +85,24 @@ __global__ void absorbed_power_kernel(const DevCloud *__restrict__ dcl, int64_t 
         const double rv = __dmul_rn((double)__ldg(C.rho + c), __ldg(C.volume + c));
         if (!(rv > 0.0)) { A_out[c] = a0; continue; }
         double acc = 0.0;
-        for (int f = 0; f < n_freq; ++f)
-            acc = __dadd_rn(acc, __dmul_rn(wf_of(s_wf, w, e_unit, f, kShared),
-                                           (double)__ldg(tally + (int64_t)f * stride + c)));
+        const long long *t = tally + c;
+        int f = 0;
+        for (; f + 4 <= n_freq; f += 4, t += 4 * stride) {
+            const long long v0 = __ldg(t), v1 = __ldg(t + stride), v2 = __ldg(t + 2 * stride), v3 = __ldg(t + 3 * stride);
+            if (plain && ((unsigned long long)(v0 | v1 | v2 | v3) >> 52) == 0ull) {
+                acc = __dadd_rn(acc, weighted_count(s_wf[f], v0));
+                acc = __dadd_rn(acc, weighted_count(s_wf[f + 1], v1));
+                acc = __dadd_rn(acc, weighted_count(s_wf[f + 2], v2));
+                acc = __dadd_rn(acc, weighted_count(s_wf[f + 3], v3));
+            } else {
+                const long long v[4] = {v0, v1, v2, v3};
+#pragma unroll 1
+                for (int k = 0; k < 4; ++k)
+                    acc = __dadd_rn(acc, __dmul_rn(wf_of(s_wf, w, e_unit, f + k, kShared), (double)v[k]));
+            }
+        }
+        for (; f < n_freq; ++f, t += stride)
+            acc = __dadd_rn(acc, __dmul_rn(wf_of(s_wf, w, e_unit, f, kShared), (double)__ldg(t)));
         A_out[c] = __dadd_rn(a0, __ddiv_rn(acc, rv));
     }
 }
