@@ -33,28 +33,47 @@ constexpr unsigned kFull = 0xffffffffu;
 
 // One package's random stream: key (seed, iteration, frequency), counter
 // (package id, block, cloud, source class); draw n = word n%4 of block n/4.
+//
+// The last two blocks and the parts of key and counter that do not change
+// lie in shared memory (12 words per thread, word j of thread t at j * 256 +
+// t: no bank conflicts), and fill() is called for the lanes of a scattering
+// together.  With one block in registers, generated at the draw that needed
+// it, nearly every draw of a scattering ran the generator for some lanes,
+// since each package stands elsewhere in its block: about five runs of 75
+// instructions where 1.4 do.
+__device__ __forceinline__ uint32_t *rng_words()
+{
+    __shared__ uint32_t s_rng[12 * 256];
+    return s_rng + threadIdx.x;
+}
+
 struct Rng {
-    uint32_t k0, k1, pid, cloud, cls, n;
-    uint32_t b0, b1, b2, b3;
+    uint32_t pid, n;
+    uint32_t have;                // words generated (a multiple of 4; n <= have <= n + 8)
 
     __device__ __forceinline__ void init(uint64_t seed, uint32_t iteration, uint32_t freq,
-                                         uint32_t pid_, uint32_t cloud_, uint32_t cls_)
+                                         uint32_t pid_, uint32_t cloud, uint32_t cls)
     {
-        k0 = (uint32_t)seed;
-        k1 = (uint32_t)(seed >> 32) ^ (iteration << 16) ^ freq;
-        pid = pid_; cloud = cloud_; cls = cls_; n = 0;
+        uint32_t *const w = rng_words();
+        w[8 * 256] = (uint32_t)seed;
+        w[9 * 256] = (uint32_t)(seed >> 32) ^ (iteration << 16) ^ freq;
+        w[10 * 256] = cloud;
+        w[11 * 256] = cls;
+        pid = pid_; n = 0; have = 0;
     }
-    __device__ __forceinline__ uint32_t next()
+    // the next block, over the one before the last: only when have - n <= 4
+    __device__ __forceinline__ void fill()
     {
-        const uint32_t j = n & 3u;
-        if (j == 0) {
-            const U4 v = philox10(pid, n >> 2, cloud, cls, k0, k1);
-            b0 = v.a; b1 = v.b; b2 = v.c; b3 = v.d;
-        }
-        ++n;
-        return j == 0 ? b0 : (j == 1 ? b1 : (j == 2 ? b2 : b3));
+        // volatile: otherwise the rounds' keys are formed ahead of the
+        // rejection loop and spill 20 registers
+        const volatile uint32_t *const k = rng_words() + 8 * 256;
+        const U4 v = philox10(pid, have >> 2, k[512], k[768], k[0], k[256]);
+        uint32_t *const b = rng_words() + ((have & 4u) << 8);
+        b[0] = v.a; b[256] = v.b; b[512] = v.c; b[768] = v.d;
+        have += 4;
     }
-    __device__ __forceinline__ float u() { return u01(next()); }
+    // a draw (its word is there: see the callers of fill)
+    __device__ __forceinline__ float u() { return u01(rng_words()[(n++ & 7u) << 8]); }
 };
 
 struct Pkg {
@@ -153,15 +172,21 @@ __device__ __forceinline__ void descend(const uint32_t *__restrict__ cells, Pkg 
 }
 
 // (cos phi, sin phi) from a point drawn uniformly in the unit disk.  After 64
-// rejections (probability < 1e-42) the azimuth 0 is used, so the loop is bounded.
+// rejections (probability < 1e-42) the azimuth 0 is used, so the loop is
+// bounded.  The words of the first try are there already, and one more.
 __device__ __forceinline__ void disk(Rng &r, float &c, float &s)
 {
     float a = 1.0f, b = 0.0f, r2 = 1.0f;
-    for (int tries = 0; tries < 64; ++tries) {
-        const float ta = __fsub_rn(__fmul_rn(2.0f, r.u()), 1.0f);
-        const float tb = __fsub_rn(__fmul_rn(2.0f, r.u()), 1.0f);
+    float ua = r.u(), ub = r.u();
+    for (int tries = 0;;) {
+        const float ta = __fsub_rn(__fmul_rn(2.0f, ua), 1.0f);
+        const float tb = __fsub_rn(__fmul_rn(2.0f, ub), 1.0f);
         const float t2 = __fadd_rn(__fmul_rn(ta, ta), __fmul_rn(tb, tb));
         if (t2 <= 1.0f && t2 > 0.0f) { a = ta; b = tb; r2 = t2; break; }
+        if (++tries == 64) break;
+        if (r.have - r.n <= 2u) r.fill();           // two draws, and one for the free path that follows
+        ua = r.u();
+        ub = r.u();
     }
     const float rr = __fsqrt_rn(r2);
     c = __fdiv_rn(a, rr);
@@ -184,6 +209,7 @@ __device__ __forceinline__ void isotropic(Rng &r, Pkg &p)
 // old direction by the azimuth from the disk sampler; renormalised.
 __device__ __forceinline__ void hg_scatter(Rng &r, float g, Pkg &p)
 {
+    if (r.have - r.n <= 4u) r.fill();               // four words: up to the first rejection, and the free path's
     const float u = r.u();
     float mu;
     if (fabsf(g) < 1e-4f) {
@@ -236,11 +262,14 @@ __device__ __forceinline__ int32_t root_cell(const DevCloud &C, int i, int j, in
 
 // Emission (Sect. 2.2 background and point sources, Sect. 3.2 dust).  Returns
 // false for a dust package of zero weight (nothing to trace).  kStack: also
-// fill the lane's ancestor rows for the cell it starts in.
+// fill the lane's ancestor rows for the cell it starts in.  At most six draws
+// up to the first rejection in disk(), and the free path's: two blocks.
 template <bool kStack>
 __device__ bool emit(const DevCloud &C, const DevItem &it, uint32_t pid, Rng &r, Pkg &p, int32_t *anc)
 {
     p.h = 1.0f;
+    r.fill();
+    r.fill();
     if (it.source == SOC_SRC_BACKGROUND) {
         const float fx = __int2float_rn(C.nx), fy = __int2float_rn(C.ny), fz = __int2float_rn(C.nz);
         const float ax = __fmul_rn(fy, fz), ay = __fmul_rn(fx, fz), az = __fmul_rn(fx, fy);
@@ -550,12 +579,12 @@ __global__ void __launch_bounds__(256, kMinBlocks) trace_kernel(const TraceParam
 
     Pkg p;
     Rng r;
+    r.pid = r.n = r.have = 0;
     p.steps = 0; p.W = 0; p.pend = 0; p.wf = 0; p.scat = false;
     bool active = false;
     int item = -1;
     float kabs = 0.f, ksca = 0.f, g = 0.f;
     unsigned long long *tally = nullptr;
-    uint64_t gidx = 0;
     // per-lane statistics, flushed when the lane moves to another item; the
     // sums live in shared memory (touched once per package) to spare registers
     __shared__ unsigned long long s_acc[4][256];     // escaped, capped, steps, emitted
@@ -606,11 +635,12 @@ __global__ void __launch_bounds__(256, kMinBlocks) trace_kernel(const TraceParam
             const bool get = !active && rank < take;
             bool moved = false;              // the lane's packages come from another item now
             int next_item = -1;
+            const uint64_t gidx = q_next + rank;
             if (get) {
-                gidx = q_next + rank;
-                const int it_idx = find_item(P.prefix, P.n_items, gidx);
-                moved = it_idx != item;
+                // mostly the item of the lane's last package
+                moved = item < 0 || gidx < P.prefix[item] || gidx >= P.prefix[item + 1];
                 if (moved) {
+                    const int it_idx = find_item(P.prefix, P.n_items, gidx);
                     const DevItem &IT = P.items[it_idx];
                     C = P.clouds + IT.cloud;
                     const float2 kap = __ldg(C->kappa + IT.freq);
@@ -702,7 +732,7 @@ __global__ void __launch_bounds__(256, kMinBlocks) trace_kernel(const TraceParam
                 if (res == kEscaped) s_acc[0][threadIdx.x] += p.W;
                 if (res == kCapped) s_acc[1][threadIdx.x] += 1;
                 s_acc[2][threadIdx.x] += p.steps;
-                if (P.pkg_steps) P.pkg_steps[gidx] = p.steps;
+                if (P.pkg_steps) P.pkg_steps[P.prefix[item] + (r.pid - P.items[item].pid_offset)] = p.steps;
                 active = false;
             }
         }
