@@ -13,9 +13,9 @@
 //             memory, operands staged by the Tensor Memory Accelerator;
 //   dgrad:    the forward kernel with the weights flipped in space and
 //             transposed in channels;
-//   wgrad:    M = C_out, N = C_in per tap, K = voxels (split over blocks
-//             that write partial sums, reduced in a fixed order), on the
-//             tcgen05 tensor cores as well.
+//   wgrad:    M = (y and z tap, C_in), N = (x tap, C_out), K = voxels (split
+//             over blocks that write partial sums, reduced in a fixed order),
+//             on the tcgen05 tensor cores as well.
 // BF16 inputs, FP32 accumulation throughout.  Every reduction (weight and
 // bias gradients, the loss) sums per-block partials in a fixed order, so a
 // training run is bit-reproducible.
@@ -77,6 +77,20 @@ __host__ __device__ constexpr uint32_t mma_idesc(int m, int n)
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
+// One lane of the (converged) warp, the same one every time.  The branch it
+// guards keeps the MMA descriptors in uniform registers: issued from
+// "lane == 0" an MMA took 72 to 214 cycles of the issuing thread, where the
+// tensor core needs 39 (N = 16) to 64 (N = 128).
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n selp.u32 %0, 1, 0, q;\n}\n" : "=r"(p));
+    return p != 0;
+}
+
+// Warp index, the same register in every lane as far as the compiler knows.
+__device__ __forceinline__ int uniform_warp() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+
 __device__ __forceinline__ bool mbar_wait(uint32_t addr, uint32_t parity)
 {
     for (uint32_t i = 0; i < (1u << 22); ++i) {
@@ -89,8 +103,8 @@ __device__ __forceinline__ bool mbar_wait(uint32_t addr, uint32_t parity)
     return false;
 }
 
-// 16-byte asynchronous copy global -> shared through L1 (the 27 taps of a
-// tile re-read most of its input); src_bytes = 0 writes zeros
+// 16-byte asynchronous copy global -> shared through L1 (the weight gradient
+// reads its output gradient at three shifts); src_bytes = 0 writes zeros
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, uint32_t src_bytes)
 {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" :: "r"(dst), "l"(src), "r"(src_bytes) : "memory");
@@ -642,260 +656,320 @@ struct WgradArgs {
     int x_stride, x_off;
     float *part;                     // [gridDim.x][Cout][27][Cin]: each block's partial sums
     int N, D, H, W, Cin, Cout;
-    long long vox_per_block;
+    // plan (wgrad_plan)
+    int by, bxk, segs, tiles_y, n_boxes;
+    int wp, bp;                      // voxels from one 8-channel group to the next in shared memory (x, gy)
+    int n_tile, a_bytes, stage_bytes, n_stages;
+    uint32_t tmem_cols;
 };
 
 // ---------------------------------------------------------------------------
 // Weight gradient on the tcgen05 tensor cores:
-//   gw[co][tap][ci] += sum_v x[v + off(tap)][ci] gy[v][co]
-// The M = 128 rows of the accumulator are (tap, input channel) pairs: a
-// block takes TT = 128 / ci_tile consecutive taps of ci_tile input channels
-// (8 taps of 16 channels, 4 of 32, 2 of 64, 1 of 128), N = n_tile output
-// channels, K = voxels (split over blocks along x; block x writes its sums to
-// partial slice x, and reduce_partials_kernel adds the slices in order, so
-// the result does not depend on block scheduling).  Both operands are
-// staged MN-major: one 16-byte global row (8 channels of one voxel) is one
-// row of a core matrix (8 K-rows of 8 consecutive M or N elements, 128
-// bytes).  Core (mn, k) of A sits at (k * 16 + mn) * 128 bytes, of B at
-// (k * n_tile / 8 + mn) * 128: the stride between cores along M/N (the
-// descriptor's stride offset) is 128 B, along K (its leading offset)
-// 16 * 128 or n_tile / 8 * 128 B.  A step covers kWgKV = 128 voxels (eight
-// MMAs with K = 16); two threads of the block's 256 share a voxel, and warps
-// 0-3 read the accumulator out.
+//   gw[co][tap][ci] += sum_u x[u][ci] gy[u - off(tap)][co]
+// (u runs over the input's voxels: outside the volume x is zero).  M = (dy,
+// channel group, dz) rows of the input, N = (dx, co), K = voxels.
+//
+// Both operands are MN-major without swizzle: 8 channels of a voxel (16
+// bytes) are one row of a core matrix, consecutive voxels are 16 bytes apart,
+// so a shift of the voxel index is a shift of the descriptor's start address
+// and needs no second copy.  A stage holds one box, by rows of bxk voxels at
+// one z:
+//   A: [by + 2 rows y'][HN channel groups][3 planes z'][wp voxels] of x,
+//   B: [by rows y][3 shifts dx][n_tile / 8 groups][bp voxels] of gy.
+// For an output row y the 9 HN groups (dy, h, dz) start (y HN 3 + g) wp voxels
+// into A: one stride, as the descriptor wants it, so an MMA takes 16 groups
+// (M = 128) against all three dx (N = 3 n_tile), and kTiles = ceil(9 HN / 16)
+// of them cover the 27 taps of 8 HN channels.  The last tile's rows past 9 HN
+// multiply whatever follows in shared memory and are not read out.
+//
+// The former kernel gathered all 27 taps of every voxel (27 copies of 16
+// bytes a channel group and a block barrier every 128 voxels): 224 us a
+// launch at batch 4, 64^3, 16 -> 16.  Here x is copied 3 (by + 2) / by times
+// and gy 3 times (mostly L1 hits).
+//
+// Warps 0-15 copy (16-byte cp.async; out-of-volume voxels are written as
+// zeros), one thread of warp 16 issues the MMAs, and warps 0-3 read the sums
+// out at the end.  The copies' address arithmetic is what bounds the kernel
+// (eight copying warps: 77 us at 64^3, 16 -> 16, against 20 us of MMAs).  A block takes the boxes [n_boxes b / chunks, n_boxes
+// (b + 1) / chunks) and writes its sums to partial slice b;
+// reduce_partials_kernel adds the slices in order, so the result does not
+// depend on scheduling.  Rows of at most 8 voxels are taken in pairs (K = 16
+// is the descriptors' two 8-voxel cores, one row apart).
 // ---------------------------------------------------------------------------
-constexpr int kWgKV = 128;
-constexpr int kWgThreads = 2 * kWgKV;         // two threads per voxel of a step
+constexpr int kWgCopyWarps = 16;
+constexpr int kWgThreads = 32 * (kWgCopyWarps + 1);
 
 __host__ __device__ constexpr uint32_t mma_idesc_mn(int m, int n)
 {
     return mma_idesc(m, n) | (1u << 15) | (1u << 16);       // A and B MN-major
 }
 
-__global__ void __launch_bounds__(kWgThreads) conv3d_wgrad_tc_kernel(const WgradArgs a, int ci_tile, int n_tile,
-                                                             uint32_t tmem_cols, int n_stages)
+__host__ __device__ constexpr int wgrad_tiles(int hn) { return (9 * hn + 15) / 16; }
+
+template <int HN>
+__global__ void __launch_bounds__(kWgThreads, 1) conv3d_wgrad_tc_kernel(const WgradArgs a)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
-    const int a_bytes = 128 * kWgKV * 2, b_bytes = n_tile * kWgKV * 2;
-    const int stage_bytes = a_bytes + b_bytes;
-    uint64_t *mbar = reinterpret_cast<uint64_t *>(smem + n_stages * stage_bytes);
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(smem + n_stages * stage_bytes + 8 * n_stages);
-    const uint32_t smem0 = smem_u32(smem);
-    const int tid = threadIdx.x, warp = tid >> 5;
-    const long long V = (long long)a.N * a.D * a.H * a.W;
-    const int TT = 128 / ci_tile;                         // taps per block
-    const int n_co_tiles = a.Cout / n_tile;
-    const int tap0 = blockIdx.y * TT;
-    const int ci0 = (blockIdx.z / n_co_tiles) * ci_tile;
-    const int co0 = (blockIdx.z % n_co_tiles) * n_tile;
-    const long long vb = (long long)blockIdx.x * a.vox_per_block;
-    const long long ve = vb + a.vox_per_block < V ? vb + a.vox_per_block : V;
-    const int total = (int)((ve - vb + kWgKV - 1) / kWgKV);
+    constexpr int kTiles = wgrad_tiles(HN);
+    const int tid = threadIdx.x, warp = uniform_warp(), lane = tid & 31;
+    const int n_stages = a.n_stages;
+    // bookkeeping first: the last stage is followed by the pad that the last
+    // tile's surplus rows may reach into
+    uint64_t *full = reinterpret_cast<uint64_t *>(smem), *empty = full + 8, *done = empty + 8;
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(done + 1);
+    int *s_fail = reinterpret_cast<int *>(tslot + 1);
+    volatile int *fail = s_fail;
+    const uint32_t smem0 = smem_u32(smem) + 256u;
 
-    if (warp == 0) {
+    if (warp == kWgCopyWarps) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                     :: "r"(smem_u32(tslot)), "r"(tmem_cols) : "memory");
+                     :: "r"(smem_u32(tslot)), "r"(a.tmem_cols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (tid == 0) {
-        for (int k = 0; k < n_stages; ++k)
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&mbar[k])) : "memory");
+        for (int k = 0; k < n_stages; ++k) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(smem_u32(&full[k])), "r"(kWgCopyWarps) : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&empty[k])) : "memory");
+        }
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(done)) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        *s_fail = 0;
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tslot;
 
-    const int NC = n_tile / 8, CP = ci_tile / 8;           // 16-byte pieces per voxel of B and per tap of A
-    const uint32_t a_lbo = 16 * 128, b_lbo = (uint32_t)NC * 128;      // stride between cores along K
-    const uint32_t idesc = mma_idesc_mn(128, n_tile);
-    const int kv = tid & (kWgKV - 1), half = tid / kWgKV;              // this thread's voxel and half
+    const int n_ci = a.Cin / (8 * HN);
+    const int ci0 = ((int)blockIdx.y % n_ci) * 8 * HN, co0 = ((int)blockIdx.y / n_ci) * a.n_tile;
+    const int box0 = (int)((long long)a.n_boxes * blockIdx.x / gridDim.x);
+    const int box1 = (int)((long long)a.n_boxes * (blockIdx.x + 1) / gridDim.x);
+    const int nn = a.n_tile / 8;                           // channel groups of gy
 
-    // this thread's 8 pieces of A: piece pc = half * 8 + i is tap tap0 +
-    // pc / CP of the block (offsets tdx, tdy, tdz), channels tco
-    int tdx[8], tdy[8], tdz[8], tco[8];
-    bool tin[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int pc = half * 8 + i, tl = pc / CP, tap = tap0 + tl;
-        tin[i] = tap < 27;
-        tdz[i] = tap / 9 - 1;
-        tdy[i] = (tap / 3) % 3 - 1;
-        tdx[i] = tap % 3 - 1;
-        tco[i] = a.x_off + ci0 + (pc - tl * CP) * 8;
-    }
-    // the voxel of the next step, advanced by kWgKV per step
-    long long cv = vb + kv;
-    int cx = 0, cy = 0, cz = 0;
-    long long cn = 0;
-    {
-        long long q = cv < V ? cv : 0;
-        cx = (int)(q % a.W); q /= a.W;
-        cy = (int)(q % a.H); q /= a.H;
-        cz = (int)(q % a.D); cn = q / a.D;
-    }
-
-    auto issue = [&](int t) {
-        if (t < total) {
-            const uint32_t st = smem0 + (uint32_t)((t % n_stages) * stage_bytes);
-            const long long v = cv;
-            const bool vin = v < ve;
-            // A: the 16 pieces of this voxel's row of cores
-            const uint32_t arow = st + (uint32_t)(((kv >> 3) * 16) * 128 + (kv & 7) * 16);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int zz = cz + tdz[i], yy = cy + tdy[i], xx = cx + tdx[i];
-                const bool ok = vin && tin[i] && (unsigned)zz < (unsigned)a.D && (unsigned)yy < (unsigned)a.H &&
-                                (unsigned)xx < (unsigned)a.W;
-                const long long sv = ok ? ((cn * a.D + zz) * a.H + yy) * a.W + xx : 0;
-                cp_async16(arow + (half * 8 + i) * 128, a.x + sv * a.x_stride + tco[i], ok ? 16u : 0u);
-            }
-            // B: gy[v][co0 .. co0 + n_tile - 1], half of the NC pieces
-            const uint32_t brow = st + (uint32_t)a_bytes + (uint32_t)(((kv >> 3) * NC) * 128 + (kv & 7) * 16);
-            for (int nc = half * (NC / 2); nc < (half + 1) * (NC / 2); ++nc)
-                cp_async16(brow + nc * 128, a.gy + (vin ? v * a.gy_stride : 0) + a.gy_off + co0 + nc * 8,
-                           vin ? 16u : 0u);
-            // next step's voxel: kWgKV further along x, carried into y, z, n
-            cv += kWgKV;
-            cx += kWgKV;
-            while (cx >= a.W) {
-                cx -= a.W;
-                if (++cy == a.H) {
-                    cy = 0;
-                    if (++cz == a.D) { cz = 0; ++cn; }
+    if (warp < kWgCopyWarps) {
+        // lane's first piece of a row of x and of gy (channel groups fastest),
+        // and what 32 pieces further on means in global and shared memory
+        const int ax = lane / HN, ah = lane % HN;
+        const uint32_t a_dst = (uint32_t)(ah * 3 * a.wp + ax) * 16u;
+        const int a_src = ax * a.x_stride + ah * 8, a_step = (32 / HN) * a.x_stride;
+        const int q0 = lane / nn, r0 = lane - q0 * nn, dq = 32 / nn, dr = 32 - dq * nn;
+        int st = 0, issued = 0, told = 0;
+        uint32_t ph = 0;
+        // the oldest box not yet announced has landed: make it visible to the
+        // tensor cores and announce it
+        auto announce = [&]() {
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0)
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_u32(&full[told % n_stages])) : "memory");
+            ++told;
+        };
+        for (int box = box0; box < box1; ++box) {
+            bool ok = !*fail;
+            if (ok && issued >= n_stages) ok = mbar_wait(smem_u32(&empty[st]), ph ^ 1u);
+            if (__any_sync(0xffffffffu, !ok)) { if (lane == 0) atomicExch(s_fail, 1); break; }
+            int q = box;
+            const int seg = q % a.segs; q /= a.segs;
+            const int ty = q % a.tiles_y; q /= a.tiles_y;
+            const int z = q % a.D, n = q / a.D;
+            const int x0 = seg * a.bxk, y0 = ty * a.by;
+            const uint32_t A0 = smem0 + (uint32_t)(st * a.stage_bytes), B0 = A0 + (uint32_t)a.a_bytes;
+            const int wx = a.W - x0;                       // voxels of the rows left from x0 on
+            const int rows = 3 * (a.by + 2);
+            for (int r = warp; r < rows; r += kWgCopyWarps) {
+                const int yp = r / 3, zp = r - 3 * yp;
+                const int yy = y0 + yp - 1, zz = z + zp - 1;
+                const bool row = (unsigned)yy < (unsigned)a.H && (unsigned)zz < (unsigned)a.D;
+                const bf16 *const base = a.x + (row ? ((((long long)n * a.D + zz) * a.H + yy) * a.W + x0) * a.x_stride : 0LL) +
+                                         a.x_off + ci0;
+                const int lim = row ? wx : 0;
+                uint32_t dst = A0 + (uint32_t)((yp * HN * 3 + zp) * a.wp) * 16u + a_dst;
+                int off = a_src;
+#pragma unroll 4
+                for (int xq = ax; xq < a.bxk; xq += 32 / HN) {
+                    const bool in = xq < lim;
+                    cp_async16(dst, base + (in ? off : 0), in ? 16u : 0u);
+                    dst += 32 / HN * 16;
+                    off += a_step;
                 }
             }
+            for (int r = warp; r < 3 * a.by; r += kWgCopyWarps) {
+                const int y = r / 3, c = r - 3 * y, yy = y0 + y;
+                const bool row = yy < a.H;
+                // shared voxel q is voxel x0 + q - (c - 1) of the row
+                const bf16 *const base = a.gy + (row ? (((long long)n * a.D + z) * a.H + yy) * a.W * a.gy_stride : 0LL) +
+                                         a.gy_off + co0;
+                const int sh = x0 - (c - 1), len = row ? a.W : 0;
+                const uint32_t dst = B0 + (uint32_t)(r * nn * a.bp) * 16u;
+#pragma unroll 4
+                for (int xq = q0, g = r0; xq < a.bxk;) {
+                    const bool in = (unsigned)(xq + sh) < (unsigned)len;
+                    cp_async16(dst + (uint32_t)(g * a.bp + xq) * 16u, base + (in ? (xq + sh) * a.gy_stride + g * 8 : 0),
+                               in ? 16u : 0u);
+                    xq += dq; g += dr;
+                    if (g >= nn) { g -= nn; ++xq; }
+                }
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+            ++issued;
+            if (++st == n_stages) { st = 0; ph ^= 1u; }
+            if (issued > 1) {
+                asm volatile("cp.async.wait_group 1;" ::: "memory");
+                announce();
+            }
         }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    };
-
-    bool ok_run = true;
-    int last = -1;
-    const int ahead = n_stages - 2;
-    for (int t = 0; t < ahead; ++t) issue(t);
-    for (int step = 0; step < total; ++step) {
-        const int s = step % n_stages;
-        const int nxt = step + ahead;
-        bool waited = true;
-        if (step >= 2 && nxt < total) {
-            const int prev = step - 2;
-            waited = mbar_wait(smem_u32(&mbar[prev % n_stages]), (uint32_t)(prev / n_stages) & 1u);
-        }
-        if (waited) issue(nxt);
-        else asm volatile("cp.async.commit_group;" ::: "memory");
-        // this step's copies have landed once at most `ahead` later groups
-        // are pending (the count is an immediate)
-        switch (ahead) {
-        case 1: asm volatile("cp.async.wait_group 1;" ::: "memory"); break;
-        case 2: asm volatile("cp.async.wait_group 2;" ::: "memory"); break;
-        case 3: asm volatile("cp.async.wait_group 3;" ::: "memory"); break;
-        case 4: asm volatile("cp.async.wait_group 4;" ::: "memory"); break;
-        case 5: asm volatile("cp.async.wait_group 5;" ::: "memory"); break;
-        default: asm volatile("cp.async.wait_group 6;" ::: "memory"); break;
-        }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        if (!__syncthreads_and(waited)) { ok_run = false; break; }
-        if (tid == 0) {
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        while (told < issued) announce();
+    } else if (elect_one()) {
+        const uint32_t idesc = mma_idesc_mn(128, 3 * a.n_tile);
+        const bool pair = a.bxk == 8;                      // two rows of 8 voxels per MMA
+        const int a_row = HN * 3 * a.wp, b_row = 3 * nn * a.bp;          // in voxels of 16 bytes
+        const uint32_t a_lbo = pair ? (uint32_t)a_row * 16u : 128u, b_lbo = pair ? (uint32_t)b_row * 16u : 128u;
+        const int row_steps = pair ? 1 : a.bxk / 16, row_inc = pair ? 2 : 1;
+        int st = 0;
+        uint32_t ph = 0, acc = 0;
+        for (int box = box0; box < box1; ++box) {
+            if (!mbar_wait(smem_u32(&full[st]), ph)) { atomicExch(s_fail, 1); break; }
+            if (*fail) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t a0 = smem0 + (uint32_t)(s * stage_bytes), b0 = a0 + (uint32_t)a_bytes;
+            const int ty = (box / a.segs) % a.tiles_y;
+            const int rows = min(a.by, a.H - ty * a.by);
+            const uint32_t A0 = smem0 + (uint32_t)(st * a.stage_bytes);
+            const uint64_t da = smem_desc(A0, a_lbo, (uint32_t)a.wp * 16u);
+            const uint64_t db = smem_desc(A0 + (uint32_t)a.a_bytes, b_lbo, (uint32_t)a.bp * 16u);
+            for (int y = 0; y < rows; y += row_inc) {
+                for (int s = 0; s < row_steps; ++s) {
+                    const uint64_t ad = da + (uint32_t)(y * a_row + s * 16), bd = db + (uint32_t)(y * b_row + s * 16);
 #pragma unroll
-            for (int j = 0; j < kWgKV / 16; ++j) {
-                const uint64_t ad = smem_desc(a0 + j * 2 * a_lbo, a_lbo, 128);
-                const uint64_t bd = smem_desc(b0 + j * 2 * b_lbo, b_lbo, 128);
-                const uint32_t acc = (step > 0 || j > 0) ? 1u : 0u;
-                asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                             " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-                             :: "r"(tmem), "l"(ad), "l"(bd), "r"(idesc), "r"(acc) : "memory");
+                    for (int t = 0; t < kTiles; ++t) {
+                        asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+                                     " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
+                                     :: "r"(tmem + (uint32_t)(t * 3 * a.n_tile)), "l"(ad + (uint32_t)(t * 16 * a.wp)),
+                                        "l"(bd), "r"(idesc), "r"(acc) : "memory");
+                    }
+                    acc = 1;
+                }
             }
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                         :: "r"(smem_u32(&mbar[s])) : "memory");
+                         :: "r"(smem_u32(&empty[st])) : "memory");
+            if (++st == n_stages) { st = 0; ph ^= 1u; }
         }
-        last = step;
+        // every MMA issued, also after a failure, has completed before the
+        // tensor memory is read and freed
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
+                     :: "r"(smem_u32(done)) : "memory");
     }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    {
-        bool done = true;
-        if (last >= 0) done = mbar_wait(smem_u32(&mbar[last % n_stages]), (uint32_t)(last / n_stages) & 1u);
-        ok_run = __syncthreads_and(ok_run && done);
-    }
+    __syncwarp();
+    const bool finished = mbar_wait(smem_u32(done), 0);
+    const bool ok_run = __syncthreads_and(finished && !*fail);
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (!ok_run) {
         if (tid == 0) atomicExch(&g_tc_error, 1);
     } else if (warp < 4) {
-        // warps 0-3 read the 128 accumulator lanes (warp w: lanes 32w ..)
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t row_addr = tmem + ((uint32_t)(warp * 32) << 16);
-        const int tap = tap0 + tid / ci_tile, ci = ci0 + tid % ci_tile;   // accumulator lane = (tap, ci)
+        // accumulator row 8 (g mod 16) + c of tile g / 16: group g = (dy HN + h) 3 + dz, channel ci0 + 8 h + c
         float *const slice = a.part + (long long)blockIdx.x * a.Cout * 27 * a.Cin;
-        for (int c = 0; c < n_tile; c += 16) {
-            uint32_t r[16];
-            asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-                         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-                           "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-                           "=r"(r[14]), "=r"(r[15])
-                         : "r"(row_addr + (uint32_t)c));
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            if (tap >= 27) continue;
-            float *dst = slice + ((long long)(co0 + c) * 27 + tap) * a.Cin + ci;
 #pragma unroll
-            for (int j = 0; j < 16; ++j) dst[(long long)j * 27 * a.Cin] = last >= 0 ? __uint_as_float(r[j]) : 0.f;
+        for (int t = 0; t < kTiles; ++t) {
+            const int g = 16 * t + tid / 8, dz = g % 3, h = (g / 3) % HN, dy = g / (3 * HN);
+            const bool valid = g < 9 * HN;
+            float *const dst = slice + (long long)((9 * dz + 3 * dy) * a.Cin + ci0 + 8 * h + tid % 8);
+            for (int dx = 0; dx < 3; ++dx)
+                for (int c = 0; c < a.n_tile; c += 16) {
+                    uint32_t r[16];
+                    tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)((3 * t + dx) * a.n_tile + c), r);
+                    if (!valid) continue;
+#pragma unroll
+                    for (int j = 0; j < 16; ++j)
+                        dst[((long long)(co0 + c + j) * 27 + dx) * a.Cin] = __uint_as_float(r[j]);
+                }
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (warp == 0) {
+    if (warp == kWgCopyWarps) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(tmem_cols) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(a.tmem_cols) : "memory");
     }
 }
 
-// out[i] += sum_{k < n_parts} part[k * n + i], k in increasing order (the
-// fixed-order reduction of per-block partial sums).
-__global__ void reduce_partials_kernel(const float *part, int n_parts, long long n, float *out)
+// out[i] += sum_{k < n_parts} part[k * n + i]: a block takes 256 / S elements;
+// thread row s of its S adds the parts s, s + S, ... in order, then the rows
+// are added in order (the same order on every run).  With one row everywhere
+// the parts of the small layers formed chains of up to 152 dependent loads.
+template <int S>
+__global__ void __launch_bounds__(256) reduce_partials_kernel(const float *part, int n_parts, long long n, float *out)
 {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        float s = 0.f;
-        for (int k = 0; k < n_parts; ++k) s += part[(long long)k * n + i];
-        out[i] += s;
+    constexpr int E = 256 / S;
+    __shared__ float s_sum[S][E + 1];
+    const int e = threadIdx.x % E, s = threadIdx.x / E;
+    const long long i = (long long)blockIdx.x * E + e;
+    float v = 0.f;
+    if (i < n) {
+#pragma unroll 8
+        for (int k = s; k < n_parts; k += S) v += part[(long long)k * n + i];
     }
+    if (S == 1) {
+        if (i < n) out[i] += v;
+        return;
+    }
+    s_sum[s][e] = v;
+    __syncthreads();
+    if (s == 0 && i < n) {
+        float t = 0.f;
+#pragma unroll
+        for (int k = 0; k < S; ++k) t += s_sum[k][e];
+        out[i] += t;
+    }
+}
+
+// Rows by size: enough threads to fill the chip (about 300 000), no more rows
+// than parts.
+inline void reduce_partials(const float *part, int n_parts, long long n, float *out, cudaStream_t s)
+{
+    if (n >= 300000 || n_parts < 8) reduce_partials_kernel<1><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(part, n_parts, n, out);
+    else if (n >= 10000 || n_parts < 32) reduce_partials_kernel<8><<<(unsigned)((n + 31) / 32), 256, 0, s>>>(part, n_parts, n, out);
+    else reduce_partials_kernel<64><<<(unsigned)((n + 3) / 4), 256, 0, s>>>(part, n_parts, n, out);
 }
 
 // Bias gradient, per block: part[blockIdx.x][c] = sum over the block's voxels
-// of gy[v][c] (BF16 gradient, dense C channels), 256 / C voxel lanes of C
-// channels each; bias_reduce_kernel adds the blocks' sums in a fixed order.
-__global__ void bias_grad_kernel(const bf16 *gy, int C, long long V, long long vox_per_block, float *part)
+// of gy[v][c] (BF16 gradient, dense C channels).  A thread takes the 8
+// channels of group threadIdx.x % (C / 8) (one 16-byte load a voxel), the
+// threads of a group every 256 / (C / 8)-th voxel; reduce_partials_kernel
+// adds the blocks' sums.
+__global__ void __launch_bounds__(256) bias_grad_kernel(const bf16 *gy, int C, long long V, long long vox_per_block,
+                                                        float *part)
 {
-    __shared__ float s_part[256];
+    __shared__ float s_part[256][9];
+    const int ng = C / 8, nv = 256 / ng, g = threadIdx.x % ng, lane_v = threadIdx.x / ng;
     const long long vb = (long long)blockIdx.x * vox_per_block;
     const long long ve = vb + vox_per_block < V ? vb + vox_per_block : V;
-    const int c = threadIdx.x % C, lane_v = threadIdx.x / C, nv = blockDim.x / C;
-    float s = 0.f;
-    if (lane_v < nv)
-        for (long long v = vb + lane_v; v < ve; v += nv) s += __bfloat162float(gy[v * C + c]);
-    s_part[threadIdx.x] = (lane_v < nv) ? s : 0.f;
-    __syncthreads();
-    if (threadIdx.x < C) {
-        float t = 0.f;
-        for (int k = 0; k < nv; ++k) t += s_part[k * C + threadIdx.x];
-        part[(long long)blockIdx.x * C + threadIdx.x] = t;
+    float sum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (lane_v < nv) {
+#pragma unroll 4
+        for (long long v = vb + lane_v; v < ve; v += nv) {
+            const uint4 u = *reinterpret_cast<const uint4 *>(gy + v * C + 8 * g);
+            const __nv_bfloat16 *h = reinterpret_cast<const __nv_bfloat16 *>(&u);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) sum[j] += __bfloat162float(h[j]);
+        }
     }
-}
-
-// gb[c] += sum over k of part[k][c], block c: thread t takes k = t, t + 256,
-// ... in order, then a fixed tree over the 256 threads (the same order on
-// every run).
-__global__ void bias_reduce_kernel(const float *part, int n_parts, int C, float *gb)
-{
-    __shared__ float s_sum[256];
-    const int c = blockIdx.x;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) s_part[threadIdx.x][j] = sum[j];
+    __syncthreads();
+    // channel c from its nv voxel lanes: 256 / C threads each take every
+    // (256 / C)-th of them, then their sums are added in order
+    const int c = threadIdx.x % C, q = threadIdx.x / C, nq = 256 / C;
     float t = 0.f;
-    for (int k = threadIdx.x; k < n_parts; k += blockDim.x) t += part[(long long)k * C + c];
-    s_sum[threadIdx.x] = t;
+    if (q < nq)
+        for (int k = q; k < nv; k += nq) t += s_part[k * ng + c / 8][c % 8];
     __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) s_sum[threadIdx.x] += s_sum[threadIdx.x + o];
-        __syncthreads();
+    if (q < nq) s_part[threadIdx.x][8] = t;
+    __syncthreads();
+    if (q == 0) {
+        t = 0.f;
+        for (int k = 0; k < nq; ++k) t += s_part[k * C + c][8];
+        part[(long long)blockIdx.x * C + c] = t;
     }
-    if (threadIdx.x == 0) gb[c] += s_sum[0];
 }
 
 // out_bf16[v][c] = (mask == null || mask[v][c] > 0) ? bf16(g[v][c]) : 0;
@@ -1468,48 +1542,97 @@ cudaError_t conv_launch(const ConvArgs &a, cudaStream_t s)
     return tma_launch<16>(a, s);
 }
 
-// Launch plan of the weight gradient: tiles and the split of the voxels into
-// `chunks` blocks along x (about 4 blocks per SM).
+// Launch plan of the weight gradient: channel tiles, box and stages, and the
+// split of the boxes into `chunks` blocks along x.
 struct WgradPlan {
-    int ci_tile = 0, n_tile = 0, tap_groups = 0;
-    long long per = 0, chunks = 0;
+    int hn = 0, n_tile = 0, combos = 0, by = 0, bxk = 0, segs = 0, wp = 0, bp = 0;
+    int a_bytes = 0, stage_bytes = 0, stages = 0, bytes = 0;
+    uint32_t cols = 0;
+    int n_boxes = 0, chunks = 0;
 };
 
-// Stages of a weight-gradient block and blocks per SM: as many stages as
-// leave room for two blocks (3 to 8), so that every block of the grid is
-// resident at once.
-inline void wgrad_stages(int n_tile, int sm_smem, int *stages, int *per_sm)
+// False where no plan fits (channel counts not multiples of 16).
+inline bool wgrad_plan(int N, int D, int H, int W, int Cin, int Cout, int sms, int blk_max, WgradPlan &p)
 {
-    const int stage_bytes = (128 + n_tile) * kWgKV * 2;
-    int st = (sm_smem / 2 - 2048) / stage_bytes;
-    st = st < 3 ? 3 : (st > 8 ? 8 : st);
-    *stages = st;
-    *per_sm = std::max(1, sm_smem / (st * stage_bytes + 8 * st + 16 + 1024));
-}
-
-inline WgradPlan wgrad_plan(long long V, int Cin, int Cout, int sms, int sm_smem = 233472)
-{
-    WgradPlan p;
-    // input-channel tile: 16, 32, 64 or 128 (dividing C_in), 128 / tile taps
-    // per block; output-channel tile: a multiple of 16, at most 128
-    p.ci_tile = 128;
-    while (p.ci_tile > 16 && Cin % p.ci_tile) p.ci_tile >>= 1;
-    p.n_tile = 128;          // at most 128: three stages of kWgKV voxels fit a block
-    while (p.n_tile > 16 && (p.n_tile > Cout || Cout % p.n_tile)) p.n_tile -= 16;
-    const int TT = 128 / p.ci_tile;
-    p.tap_groups = (27 + TT - 1) / TT;
-    const long long tiles = (long long)p.tap_groups * (Cin / p.ci_tile) * (Cout / p.n_tile);
-    // one wave: the voxels split into as many chunks as the SMs hold blocks
-    // of every tile
-    int stages = 0, per_sm = 0;
-    wgrad_stages(p.n_tile, sm_smem, &stages, &per_sm);
-    long long chunks = std::max(1LL, (long long)per_sm * sms / tiles);
-    long long per = (V + chunks - 1) / chunks;
-    per = (per + kWgKV - 1) / kWgKV * kWgKV;
-    if (per < kWgKV) per = kWgKV;
-    p.per = per;
-    p.chunks = (V + per - 1) / per;
-    return p;
+    if (Cin % 16 || Cout % 16) return false;
+    // Rows of at most 8 voxels go in pairs; longer ones in segments of at
+    // most 64 voxels, a multiple of 16.
+    p.segs = (W + 63) / 64;
+    p.bxk = W <= 8 ? 8 : ((W + p.segs - 1) / p.segs + 15) / 16 * 16;
+    p.segs = (W + p.bxk - 1) / p.bxk;
+    const bool pair = p.bxk == 8;
+    // group pitches for which the 8 lanes of a quarter warp (channel groups
+    // fastest) write to distinct 16-byte banks: one group apart is 128 /
+    // groups bytes modulo 128 (x: three pitches)
+    auto pitch = [&](int groups) {
+        const int want = groups == 2 ? 4 : groups == 4 ? 2 : 1;          // an odd multiple of this many banks
+        int v = p.bxk;
+        while (v % want || (v / want) % 2 == 0) ++v;
+        return v;
+    };
+    auto sizes = [&](int hn, int nt, int by) {
+        p.wp = pitch(hn);
+        p.bp = pitch(nt / 8);
+        p.a_bytes = (by + 2) * hn * 3 * p.wp * 16;
+        p.stage_bytes = (p.a_bytes + by * 3 * (nt / 8) * p.bp * 16 + 127) / 128 * 128;
+        const int pad = (wgrad_tiles(hn) * 16 - 9 * hn) * p.wp * 16;     // what the last tile reads past its groups
+        p.stages = std::min(6, (blk_max - 256 - pad) / p.stage_bytes);
+        p.bytes = 256 + p.stages * p.stage_bytes + pad;
+        p.by = by;
+        return p.stages >= 3;                // copies of one box, one landing, MMAs of one
+    };
+    // Chunks: what a tiling into 128 (tap, ci) rows by up to 128 co gives one
+    // wave of (n16 tiles: two blocks per SM).  The tensor cores' FP32
+    // accumulation truncates, so a sum depends systematically on the length
+    // of its chain: halving the chunks at batch 4, 64^3 moves the 16 -> 16
+    // layers' gradients by 1.7e-5 and the 48 -> 16 layer's by 6e-5.  Fewer
+    // where the partial sums, written once and read once, would cost more
+    // than the MMAs they spread.
+    const long long V = (long long)N * D * H * W;
+    int ci = 128, co = 128;
+    while (ci > 16 && Cin % ci) ci >>= 1;
+    while (co > 16 && (co > Cout || Cout % co)) co -= 16;
+    const long long tiles128 = (long long)((27 * ci + 127) / 128) * (Cin / ci) * (Cout / co);
+    long long chunks = std::max(1LL, (co == 16 ? 2LL : 1LL) * sms / tiles128);
+    const double steps = (double)N * D * H * p.segs * (pair ? 0.5 : p.bxk / 16);       // MMAs per tile, all chunks
+    const double part = 2.0 * 4.0 * 27.0 * Cin * Cout / 4e12;                           // s per chunk
+    const double work = steps * 27.0 * Cin * Cout / (128.0 * 128.0) * 64.0 / (2e9 * 0.5);  // s on one SM
+    const long long best_chunks = std::max(1LL, (long long)std::sqrt(work / part));
+    // (chains of at most 512 MMAs are within 1e-5 of any shorter ones)
+    chunks = steps / chunks <= 512.0 ? best_chunks : std::min(chunks, best_chunks);
+    // Channel tiles (8 hn of x, n_tile of gy), one block per SM: the least of
+    // the estimated times over the ones whose accumulators fit tensor memory.
+    // An MMA of N = 3 n_tile takes about 36 + N / 6 cycles (its operands from
+    // shared memory; measured 39, 44 and 64 at N = 16, 48 and 128), or N / 2
+    // where that is longer; a warp's 16-byte copies take about 20 cycles; L2
+    // delivers about 6 TB/s in 32-byte sectors.
+    const int step = pair ? 2 : 1;
+    double best = 0.0;
+    for (int hn = 1; hn <= 8; hn *= 2) {
+        if (Cin % (8 * hn)) continue;
+        for (int nt = 16; nt <= 80; nt += 16) {
+            if (Cout % nt || wgrad_tiles(hn) * 3 * nt > 512 || !sizes(hn, nt, step)) continue;
+            const long long combos = (long long)(Cin / (8 * hn)) * (Cout / nt), blocks = combos * chunks;
+            const double waves = (double)((blocks + sms - 1) / sms);
+            const double mma = steps / chunks * wgrad_tiles(hn) * std::max(1.5 * nt, 36.0 + 0.5 * nt) / 2e9;
+            const double copy = (double)V / chunks * (4.2 * hn + 0.375 * nt) / 32.0 * 20.0 / 2e9;
+            const double l2 = (double)V * combos * (4.2 * std::max(16 * hn, 32) + std::max(2 * nt, 32)) / 6e12;
+            const double cost = std::max(waves * std::max(mma, copy), l2);
+            if (best == 0.0 || cost < best) { best = cost; p.hn = hn; p.n_tile = nt; }
+        }
+    }
+    if (best == 0.0) return false;
+    p.combos = (Cin / (8 * p.hn)) * (Cout / p.n_tile);
+    p.cols = 32;
+    while ((int)p.cols < wgrad_tiles(p.hn) * 3 * p.n_tile) p.cols <<= 1;
+    // box height: the largest up to 8 that leaves room for 3 stages
+    int by = std::min(8, (H + step - 1) / step * step);
+    while (!sizes(p.hn, p.n_tile, by)) by -= step;
+    const long long boxes = (long long)N * D * ((H + p.by - 1) / p.by) * p.segs;
+    if (boxes > INT32_MAX) return false;
+    p.n_boxes = (int)boxes;
+    p.chunks = (int)std::min(chunks, boxes);
+    return true;
 }
 
 inline int device_sms()
@@ -1520,65 +1643,70 @@ inline int device_sms()
     return sms;
 }
 
-// Floats of partial sums a weight gradient of this shape needs.
-inline long long wgrad_part_floats(long long V, int Cin, int Cout, int sms)
+inline int device_block_smem()
 {
-    int dev = 0, sm_smem = 0;
+    int dev = 0, v = 0;
     cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-    return wgrad_plan(V, Cin, Cout, sms, sm_smem).chunks * Cout * 27LL * Cin;
+    cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    return v;
 }
 
-// gw[Cout][27][Cin] += sum_v gy[v] x[v + tap]: partial sums per voxel chunk
-// into part (part_floats available), then their ordered sum into gw.
-cudaError_t wgrad_launch(const WgradArgs &a0, float *gw, long long part_floats, cudaStream_t s)
+// Floats of partial sums a weight gradient of this shape needs.
+inline long long wgrad_part_floats(int N, int D, int H, int W, int Cin, int Cout)
 {
-    WgradArgs a = a0;
-    const long long V = (long long)a.N * a.D * a.H * a.W;
-    int dev = 0, sm_smem = 0, blk_max = 0;
-    cudaGetDevice(&dev);
-    const int sms = device_sms();
-    cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-    cudaDeviceGetAttribute(&blk_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    const WgradPlan p = wgrad_plan(V, a.Cin, a.Cout, sms, sm_smem);
-    if (a.Cin % p.ci_tile) return cudaErrorInvalidValue;
-    const long long n_w = (long long)a.Cout * 27 * a.Cin;
-    if (p.chunks * n_w > part_floats) return cudaErrorInvalidValue;
-    a.vox_per_block = p.per;
-    uint32_t cols = 32;
-    while ((int)cols < p.n_tile) cols <<= 1;
-    const int stage_bytes = (128 + p.n_tile) * kWgKV * 2;
-    int stages = 0, per_sm = 0;
-    wgrad_stages(p.n_tile, sm_smem, &stages, &per_sm);
-    const int need = stages * stage_bytes + 8 * stages + 16;
-    const int max_blocks = 512 / (int)cols;
-    const int pad = sm_smem / (max_blocks + 1) + 1024;
-    int bytes = need > pad ? need : pad;
-    if (need > blk_max) return cudaErrorInvalidValue;
-    if (bytes > blk_max) bytes = blk_max;
-    cudaError_t e = cudaFuncSetAttribute(conv3d_wgrad_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    WgradPlan p;
+    if (!wgrad_plan(N, D, H, W, Cin, Cout, device_sms(), device_block_smem(), p)) return 0;
+    return (long long)p.chunks * Cout * 27 * Cin;
+}
+
+template <int HN>
+cudaError_t wgrad_start(const WgradArgs &a, const WgradPlan &p, cudaStream_t s)
+{
+    cudaError_t e = cudaFuncSetAttribute(conv3d_wgrad_tc_kernel<HN>, cudaFuncAttributeMaxDynamicSharedMemorySize, p.bytes);
     if (e != cudaSuccess) return e;
-    dim3 grid((unsigned)p.chunks, (unsigned)p.tap_groups, (unsigned)((a.Cin / p.ci_tile) * (a.Cout / p.n_tile)));
-    conv3d_wgrad_tc_kernel<<<grid, kWgThreads, bytes, s>>>(a, p.ci_tile, p.n_tile, cols, stages);
-    reduce_partials_kernel<<<grid_1d(n_w), 256, 0, s>>>(a.part, (int)p.chunks, n_w, gw);
+    conv3d_wgrad_tc_kernel<HN><<<dim3((unsigned)p.chunks, (unsigned)p.combos), kWgThreads, p.bytes, s>>>(a);
     return cudaGetLastError();
 }
 
-// Voxels per block of the bias gradient: 16 per voxel lane of its 256 threads
-inline long long bias_vox(int C) { return 16LL * (256 / (C < 1 ? 1 : C)); }
+// gw[Cout][27][Cin] += sum_v gy[v] x[v + tap]: partial sums per chunk of
+// boxes into part (part_floats available), then their ordered sum into gw.
+cudaError_t wgrad_launch(const WgradArgs &a0, float *gw, long long part_floats, cudaStream_t s)
+{
+    WgradArgs a = a0;
+    WgradPlan p;
+    if (!wgrad_plan(a.N, a.D, a.H, a.W, a.Cin, a.Cout, device_sms(), device_block_smem(), p)) return cudaErrorInvalidValue;
+    const long long n_w = (long long)a.Cout * 27 * a.Cin;
+    if (p.chunks * n_w > part_floats) return cudaErrorInvalidValue;
+    a.by = p.by; a.bxk = p.bxk; a.segs = p.segs; a.tiles_y = (a.H + p.by - 1) / p.by; a.n_boxes = p.n_boxes;
+    a.wp = p.wp; a.bp = p.bp; a.n_tile = p.n_tile; a.a_bytes = p.a_bytes; a.stage_bytes = p.stage_bytes;
+    a.n_stages = p.stages; a.tmem_cols = p.cols;
+    const cudaError_t e = p.hn == 8 ? wgrad_start<8>(a, p, s) : p.hn == 4 ? wgrad_start<4>(a, p, s)
+                        : p.hn == 2 ? wgrad_start<2>(a, p, s) : wgrad_start<1>(a, p, s);
+    if (e != cudaSuccess) return e;
+    reduce_partials(a.part, p.chunks, n_w, gw, s);
+    return cudaGetLastError();
+}
 
-inline long long bias_part_floats(long long V, int C) { return (V + bias_vox(C) - 1) / bias_vox(C) * C; }
+// Voxels per block of the bias gradient: at least 16 per voxel lane, and at
+// most about 600 blocks (4 per SM), so that few partial sums are left.
+inline long long bias_vox(long long V, int C)
+{
+    const long long lanes = 256 / (C / 8);
+    return std::max(16 * lanes, (V + 607) / 608);
+}
+
+inline long long bias_part_floats(long long V, int C) { return (V + bias_vox(V, C) - 1) / bias_vox(V, C) * C; }
 
 // gb[C] += sum_v gy[v]: per-block sums into part, then their sum in a fixed
 // order.
 cudaError_t bias_grad_launch(const bf16 *gy, int C, long long V, float *gb, float *part, long long part_floats,
                              cudaStream_t s)
 {
-    if (C < 1 || C > 256) return cudaErrorInvalidValue;
-    const long long blocks = (V + bias_vox(C) - 1) / bias_vox(C);
+    if (C < 8 || C % 8 || C > 256) return cudaErrorInvalidValue;
+    const long long vox = bias_vox(V, C), blocks = (V + vox - 1) / vox;
     if (blocks * C > part_floats || blocks > 0x7FFFFFFF) return cudaErrorInvalidValue;
-    bias_grad_kernel<<<(unsigned)blocks, 256, 0, s>>>(gy, C, V, bias_vox(C), part);
-    bias_reduce_kernel<<<C, 256, 0, s>>>(part, (int)blocks, C, gb);
+    bias_grad_kernel<<<(unsigned)blocks, 256, 0, s>>>(gy, C, V, vox, part);
+    reduce_partials(part, (int)blocks, C, gb, s);
     return cudaGetLastError();
 }
 
@@ -1855,12 +1983,11 @@ soc_status soc_unet_create(int device, int batch, int side, int n_inputs, int *n
     A(n->g_p0, n->V1 * 16); A(n->g_e0a, n->V0 * 16); A(n->gstage, n->V0 * 48); A(n->loss, 1);
     A(n->loss_part, (size_t)grid_1d(n->V0));
     {   // partial sums: the largest weight (or bias) gradient of any layer
-        const int sms = device_sms();
         long long need = 0;
         for (int l = 0; l < kLayers; ++l) {
             const int lev = l < 2 ? 0 : l < 4 ? 1 : l < 6 ? 2 : l < 8 ? 3 : l < 10 ? 2 : l < 12 ? 1 : 0;
             const long long V = n->V0 >> (3 * lev);
-            need = std::max(need, wgrad_part_floats(V, kSpec[l].cin, kSpec[l].cout, sms));
+            need = std::max(need, wgrad_part_floats(batch, side >> lev, side >> lev, side >> lev, kSpec[l].cin, kSpec[l].cout));
             need = std::max(need, bias_part_floats(V, kSpec[l].cout));
         }
         A(n->part, (size_t)need);
@@ -2034,7 +2161,7 @@ soc_status soc_nn_conv3d_wgrad(const void *gy, const void *x, int N, int D, int 
     if (!gy || !x || !gw || Cin % 16 || Cout % 16 || N < 1 || D < 1 || H < 1 || W < 1) return SOC_ERR_ARG;
     cudaStream_t s = (cudaStream_t)stream;
     const long long V = (long long)N * D * H * W;
-    const long long need = std::max(wgrad_part_floats(V, Cin, Cout, device_sms()), bias_part_floats(V, Cout));
+    const long long need = std::max(wgrad_part_floats(N, D, H, W, Cin, Cout), bias_part_floats(V, Cout));
     // partial sums in a library-owned workspace of this device (grown on
     // demand; calls on one device share it and are ordered by the caller)
     static std::mutex ws_mutex;
