@@ -285,13 +285,13 @@ __device__ __forceinline__ void conv_producer_tail(const ConvBlock &c, int n_sta
 // error flag.  Every thread calls it.
 __device__ __forceinline__ void conv_block_end(const ConvBlock &c, uint32_t tmem_cols)
 {
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = uniform_warp();
     __syncwarp();
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     const bool ok = __syncthreads_and(!*reinterpret_cast<volatile int *>(c.s_fail));
     if (!ok) {
         if (tid == 0) atomicExch(&g_tc_error, 1);
-        if (warp == 5 && lane == 0) {
+        if (warp == 5 && elect_one()) {
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
                          :: "r"(smem_u32(c.drain)) : "memory");
             mbar_wait(smem_u32(c.drain), 0);
@@ -334,7 +334,7 @@ __global__ void __launch_bounds__(kConvThreads) conv3d_tma_kernel(const __grid_c
     volatile int *fail = s_fail;
     const uint32_t tmem = cb.tmem;
     const uint32_t smem0 = smem_u32(smem);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = uniform_warp();
     const int n0 = blockIdx.y * n_tile;
     const int n_chunks = a.Cin / KC;
     const int steps = 27 * n_chunks;                   // per box
@@ -343,7 +343,7 @@ __global__ void __launch_bounds__(kConvThreads) conv3d_tma_kernel(const __grid_c
 
 
     if (warp == 4) {
-        if (lane == 0) {
+        if (elect_one()) {
             asm volatile("prefetch.tensormap [%0];" :: "l"(reinterpret_cast<uint64_t>(&map_in)) : "memory");
             asm volatile("prefetch.tensormap [%0];" :: "l"(reinterpret_cast<uint64_t>(&map_w)) : "memory");
             // producer: step g = (box, tap, chunk) into stage st = g mod
@@ -383,7 +383,7 @@ __global__ void __launch_bounds__(kConvThreads) conv3d_tma_kernel(const __grid_c
             conv_producer_tail(cb, n_stages, issued);
         }
     } else if (warp == 5) {
-        if (lane == 0) {
+        if (elect_one()) {
             // MMA issuer: box i into accumulator i % 2, once the epilogue has
             // drained box i - 2 from it
             const uint32_t idesc = mma_idesc(128, n_tile);
@@ -496,14 +496,14 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv3d_slab_kernel(const __gr
     volatile int *fail = s_fail;
     const uint32_t tmem = cb.tmem;
     const uint32_t smem0 = smem_u32(smem);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = uniform_warp();
     const int n0 = blockIdx.y * n_tile;
     const int n_boxes = a.tiles_y * a.tiles_z * a.N;
     const uint32_t tx_bytes = (uint32_t)rows_s * kRow + 9u * (uint32_t)tap_bytes;
 
 
     if (warp == 4) {
-        if (lane == 0) {
+        if (elect_one()) {
             asm volatile("prefetch.tensormap [%0];" :: "l"(reinterpret_cast<uint64_t>(&map_in)) : "memory");
             asm volatile("prefetch.tensormap [%0];" :: "l"(reinterpret_cast<uint64_t>(&map_w)) : "memory");
             const int n_rows = (a.by + 2) * (a.bz + 2), row_bytes = bx * kRow;
@@ -545,7 +545,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv3d_slab_kernel(const __gr
             conv_producer_tail(cb, n_stages, issued);
         }
     } else if (warp == 5) {
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t idesc = mma_idesc(128, n_tile);
             const int steps = 3 * (a.Cin / KC);
             // descriptor start-address offsets (16-byte units): A rows of
