@@ -47,6 +47,8 @@ struct ConvArgs {
     int out_stride, out_off;
     int N, D, H, W, Cin, Cout;
     int relu, accumulate;           // accumulate: FP32 output += result
+    const bf16 *mask;               // see ConvOut
+    int m_stride, m_off, first_only;
 };
 
 // ---------------------------------------------------------------------------
@@ -126,12 +128,17 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, uint32
 // its loads and MMAs in flight, frees its tensor memory and returns).
 // ---------------------------------------------------------------------------
 // Output of a convolution: bias, ReLU, then BF16 or FP32 (optionally added
-// to what is there) at out[v * out_stride + out_off + co].
+// to what is there) at out[v * out_stride + out_off + co].  mask (BF16
+// output): the value is kept where mask[v * m_stride + m_off + co] > 0 and 0
+// elsewhere (an input gradient leaves through the ReLU of the layer before).
+// first_only (FP32 output): channel 0 alone, at out_f32[v].
 struct ConvOut {
     bf16 *out;
     float *out_f32;
     const float *bias;
     int out_stride, out_off, relu, accumulate;
+    const bf16 *mask;
+    int m_stride, m_off, first_only;
 };
 
 struct TmaConvArgs {
@@ -152,6 +159,33 @@ __device__ __forceinline__ void tmem_ld16(uint32_t addr, uint32_t (&rr)[16])
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+// val[j] = 0 where mask[j] is not > 0 (8 values of a 16-byte aligned mask)
+__device__ __forceinline__ void apply_mask8(const bf16 *mask, float *val)
+{
+    const uint4 m = *reinterpret_cast<const uint4 *>(mask);
+    const __nv_bfloat16 *mh = reinterpret_cast<const __nv_bfloat16 *>(&m);
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+        if (!(__bfloat162float(mh[j]) > 0.f)) val[j] = 0.f;
+}
+__device__ __forceinline__ void apply_mask16(const bf16 *mask, float *val)
+{
+    apply_mask8(mask, val);
+    apply_mask8(mask + 8, val + 8);
+}
+
+// 8 BF16 values as one 16-byte word
+__device__ __forceinline__ uint4 pack8(const float *val)
+{
+    uint32_t pk[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const __nv_bfloat162 h2 = __floats2bfloat162_rn(val[2 * j], val[2 * j + 1]);
+        pk[j] = *reinterpret_cast<const uint32_t *>(&h2);
+    }
+    return make_uint4(pk[0], pk[1], pk[2], pk[3]);
+}
+
 // Output channels co .. co + 15 of voxel v from their FP32 accumulators
 __device__ __forceinline__ void store_row16(const ConvOut &o, long long v, int co, const uint32_t (&rr)[16])
 {
@@ -163,6 +197,11 @@ __device__ __forceinline__ void store_row16(const ConvOut &o, long long v, int c
         if (o.relu) t = fmaxf(t, 0.f);
         val[j] = t;
     }
+    if (o.first_only) {
+        if (co == 0) o.out_f32[v] = val[0];
+        return;
+    }
+    if (o.mask) apply_mask16(o.mask + v * o.m_stride + o.m_off + co, val);
     const long long off = v * o.out_stride + o.out_off + co;
     if (o.out_f32) {
         float4 *dst = reinterpret_cast<float4 *>(o.out_f32 + off);
@@ -176,15 +215,9 @@ __device__ __forceinline__ void store_row16(const ConvOut &o, long long v, int c
             dst[q4] = w4;
         }
     } else {
-        uint32_t pk[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const __nv_bfloat162 h2 = __floats2bfloat162_rn(val[2 * j], val[2 * j + 1]);
-            pk[j] = *reinterpret_cast<const uint32_t *>(&h2);
-        }
         uint4 *dst = reinterpret_cast<uint4 *>(o.out + off);
-        dst[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-        dst[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+        dst[0] = pack8(val);
+        dst[1] = pack8(val + 8);
     }
 }
 
@@ -638,15 +671,21 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv3d_slab_kernel(const __gr
 }
 
 // Wt[ci][t][co] = W[co][26 - t][ci]: weights of the transposed convolution.
-__global__ void flip_weights_kernel(const bf16 *W, int Cout, int Cin, bf16 *Wt)
+template <class Int>
+__device__ __forceinline__ void flip_weights(const bf16 *W, Int Cout, Int Cin, bf16 *Wt)
 {
-    const long long n = (long long)Cout * 27 * Cin;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int co = (int)(i % Cout);
-        const int t = (int)((i / Cout) % 27);
-        const int ci = (int)(i / (27LL * Cout));
+    const Int n = Cout * 27 * Cin;
+    for (Int i = blockIdx.x * (Int)blockDim.x + threadIdx.x; i < n; i += (Int)gridDim.x * blockDim.x) {
+        const Int co = i % Cout, q = i / Cout, t = q % 27, ci = q / 27;
         Wt[i] = W[((long long)co * 27 + (26 - t)) * Cin + ci];
     }
+}
+
+__global__ void flip_weights_kernel(const bf16 *W, int Cout, int Cin, bf16 *Wt)
+{
+    // 32-bit index arithmetic where it is enough (the divisions are the cost)
+    if ((long long)Cout * 27 * Cin < (1LL << 30)) flip_weights<unsigned>(W, (unsigned)Cout, (unsigned)Cin, Wt);
+    else flip_weights<long long>(W, Cout, Cin, Wt);
 }
 
 struct WgradArgs {
@@ -972,36 +1011,6 @@ __global__ void __launch_bounds__(256) bias_grad_kernel(const bf16 *gy, int C, l
     }
 }
 
-// out_bf16[v][c] = (mask == null || mask[v][c] > 0) ? bf16(g[v][c]) : 0;
-// one voxel per thread, 8 channels at a time (C, the strides and offsets
-// multiples of 8, of 4 for g).
-__global__ void mask_to_bf16_kernel(const float *g, int g_stride, int g_off, const bf16 *mask, int m_stride, int m_off,
-                                    int C, long long V, bf16 *out)
-{
-    const long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (v >= V) return;
-    const float *gv = g + v * g_stride + g_off;
-    for (int c = 0; c < C; c += 8) {
-        const float4 a = *reinterpret_cast<const float4 *>(gv + c);
-        const float4 b = *reinterpret_cast<const float4 *>(gv + c + 4);
-        float val[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-        if (mask) {
-            const uint4 m = *reinterpret_cast<const uint4 *>(mask + v * m_stride + m_off + c);
-            const __nv_bfloat16 *mh = reinterpret_cast<const __nv_bfloat16 *>(&m);
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-                if (!(__bfloat162float(mh[j]) > 0.f)) val[j] = 0.f;
-        }
-        uint32_t pk[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const __nv_bfloat162 h2 = __floats2bfloat162_rn(val[2 * j], val[2 * j + 1]);
-            pk[j] = *reinterpret_cast<const uint32_t *>(&h2);
-        }
-        *reinterpret_cast<uint4 *>(out + v * C + c) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-    }
-}
-
 // Kernels over the voxels of a volume N x D x H x W: blockIdx.y (strided by
 // gridDim.y) walks the rows (n, z, y), threads the row's voxels x times
 // channel groups of 8 (BF16) or 4 (FP32).
@@ -1044,11 +1053,16 @@ __global__ void maxpool_kernel(const bf16 *in, int in_stride, int in_off, int N,
     }
 }
 
-// g_in[argmax] += g_out (FP32; g_in strided view of the fine grid).  Coarse
-// rows; the 8 voxels of an octant belong to one coarse voxel, so no two
-// threads write one element.
-__global__ void maxpool_bwd_kernel(const float *g_out, const uint8_t *arg, int N, int D, int H, int W, int C, float *g_in,
-                                   int in_stride, int in_off)
+// Gradient of a pooled layer, through its ReLU: out[fine] = bf16(mask > 0 ?
+// g_skip[fine] + (fine is the argmax of its octant ? g_out[coarse] : nothing)
+// : 0), g_skip a strided FP32 view of the fine grid (the skip connection's
+// gradient), mask the layer's output (strided BF16 view), out dense.  Coarse
+// rows; the 8 voxels of an octant belong to one coarse voxel.  Adding into
+// g_skip and masking it in a second kernel moved the fine FP32 gradient
+// three times more.
+__global__ void maxpool_bwd_kernel(const float *g_out, const uint8_t *arg, int N, int D, int H, int W, int C,
+                                   const float *g_skip, int s_stride, int s_off, const bf16 *mask, int m_stride,
+                                   int m_off, bf16 *out)
 {
     const int d2 = D / 2, h2 = H / 2, w2 = W / 2, ng = C / 8;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1063,10 +1077,17 @@ __global__ void maxpool_bwd_kernel(const float *g_out, const uint8_t *arg, int N
         const float4 g1 = *reinterpret_cast<const float4 *>(g_out + ov * C + c + 4);
         const float gv[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int o = (int)(((j < 4 ? a.x : a.y) >> (8 * (j & 3))) & 0xFFu);
+        for (int o = 0; o < 8; ++o) {
             const int zz = 2 * z + (o >> 2), yy = 2 * y + ((o >> 1) & 1), xx = 2 * x + (o & 1);
-            g_in[((((long long)n * D + zz) * H + yy) * W + xx) * in_stride + in_off + c + j] += gv[j];
+            const long long v = (((long long)n * D + zz) * H + yy) * W + xx;
+            const float4 s0 = *reinterpret_cast<const float4 *>(g_skip + v * s_stride + s_off + c);
+            const float4 s1 = *reinterpret_cast<const float4 *>(g_skip + v * s_stride + s_off + c + 4);
+            float val[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if ((int)(((j < 4 ? a.x : a.y) >> (8 * (j & 3))) & 0xFFu) == o) val[j] += gv[j];
+            apply_mask8(mask + v * m_stride + m_off + c, val);
+            *reinterpret_cast<uint4 *>(out + v * C + c) = pack8(val);
         }
     }
 }
@@ -1088,26 +1109,32 @@ __global__ void upsample_kernel(const bf16 *in, int N, int d2, int h2, int w2, i
     }
 }
 
-// g_in[coarse] = sum over the 8 fine voxels, in octant order, of g_out
-// (strided FP32 view).  Coarse rows, 4 channels per thread.
+// Gradient of an upsampled layer, through its ReLU: out[coarse] = bf16(mask >
+// 0 ? sum over the 8 fine voxels, in octant order, of g_out : 0), g_out a
+// strided FP32 view, mask the layer's output and out dense BF16.  Coarse
+// rows, 8 channels per thread.
 __global__ void upsample_bwd_kernel(const float *g_out, int out_stride, int out_off, int N, int d2, int h2, int w2, int C,
-                                    float *g_in)
+                                    const bf16 *mask, bf16 *out)
 {
-    const int D = 2 * d2, H = 2 * h2, W = 2 * w2, ng = C / 4;
+    const int D = 2 * d2, H = 2 * h2, W = 2 * w2, ng = C / 8;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= w2 * ng) return;
-    const int x = t / ng, c = (t - x * ng) * 4;
+    const int x = t / ng, c = (t - x * ng) * 8;
     const int rows = N * d2 * h2;
     for (int row = blockIdx.y; row < rows; row += gridDim.y) {
         const int y = row % h2, q = row / h2, z = q % d2, n = q / d2;
-        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+        float val[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
         for (int o = 0; o < 8; ++o) {
             const int zz = 2 * z + (o >> 2), yy = 2 * y + ((o >> 1) & 1), xx = 2 * x + (o & 1);
-            const float4 g = *reinterpret_cast<const float4 *>(
-                g_out + ((((long long)n * D + zz) * H + yy) * W + xx) * out_stride + out_off + c);
-            s.x += g.x; s.y += g.y; s.z += g.z; s.w += g.w;
+            const float *g = g_out + ((((long long)n * D + zz) * H + yy) * W + xx) * out_stride + out_off + c;
+            const float4 a = *reinterpret_cast<const float4 *>(g), b = *reinterpret_cast<const float4 *>(g + 4);
+            val[0] += a.x; val[1] += a.y; val[2] += a.z; val[3] += a.w;
+            val[4] += b.x; val[5] += b.y; val[6] += b.z; val[7] += b.w;
         }
-        *reinterpret_cast<float4 *>(g_in + ((long long)row * w2 + x) * C + c) = s;
+        const long long v = (long long)row * w2 + x;
+        apply_mask8(mask + v * C + c, val);
+        *reinterpret_cast<uint4 *>(out + v * C + c) = pack8(val);
     }
 }
 
@@ -1120,33 +1147,25 @@ __global__ void input_kernel(const float *in, long long V, int n_in, bf16 *x16)
     float val[16];
 #pragma unroll
     for (int c = 0; c < 16; ++c) val[c] = c < n_in ? in[v * n_in + c] : 0.f;
-    uint32_t pk[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        const __nv_bfloat162 h2 = __floats2bfloat162_rn(val[2 * j], val[2 * j + 1]);
-        pk[j] = *reinterpret_cast<const uint32_t *>(&h2);
-    }
     uint4 *dst = reinterpret_cast<uint4 *>(x16 + v * 16);
-    dst[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-    dst[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+    dst[0] = pack8(val);
+    dst[1] = pack8(val + 8);
 }
 
-// Prediction = head channel 0; MSE loss and its gradient into head channel 0.
-// loss_part[blockIdx.x] = the block's share of the loss (sum_loss_kernel
-// adds the shares in order).
-__global__ void mse_kernel(const float *head, const float *target, long long V, float *pred, float *ghead,
-                           double *loss_part)
+// MSE loss of the prediction and its gradient, BF16, in channel 0 of the 16
+// the head's layer has (the others zero).  loss_part[blockIdx.x] = the
+// block's share of the loss (sum_loss_kernel adds the shares in order).
+__global__ void mse_kernel(const float *pred, const float *target, long long V, bf16 *ghead, double *loss_part)
 {
     __shared__ double part[256];
     double s = 0.0;
     for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < V; v += (long long)gridDim.x * blockDim.x) {
-        const float p = head[v * 16];
-        if (pred) pred[v] = p;
-        if (target) {
-            const float d = p - target[v];
-            s += (double)d * d;
-            if (ghead) ghead[v * 16] = 2.0f * d / (float)V;
-        }
+        const float d = pred[v] - target[v];
+        s += (double)d * d;
+        const float val[8] = {2.0f * d / (float)V, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        uint4 *dst = reinterpret_cast<uint4 *>(ghead + v * 16);
+        dst[0] = pack8(val);
+        dst[1] = make_uint4(0u, 0u, 0u, 0u);
     }
     part[threadIdx.x] = s;
     __syncthreads();
@@ -1154,7 +1173,7 @@ __global__ void mse_kernel(const float *head, const float *target, long long V, 
         if (threadIdx.x < o) part[threadIdx.x] += part[threadIdx.x + o];
         __syncthreads();
     }
-    if (threadIdx.x == 0 && loss_part && target) loss_part[blockIdx.x] = part[0] / (double)V;
+    if (threadIdx.x == 0) loss_part[blockIdx.x] = part[0] / (double)V;
 }
 
 // loss = sum of the blocks' shares: thread t takes k = t, t + 256, ... in
@@ -1334,7 +1353,8 @@ cudaError_t tma_launch(const ConvArgs &a, cudaStream_t s)
     t.tiles_y = (a.H + t.by - 1) / t.by;
     t.tiles_z = (a.D + t.bz - 1) / t.bz;
     const long long tiles = (long long)t.tiles_x * t.tiles_y * t.tiles_z * ((a.N + t.bn - 1) / t.bn);
-    t.o = ConvOut{a.out, a.out_f32, a.bias, a.out_stride, a.out_off, a.relu, a.accumulate};
+    t.o = ConvOut{a.out, a.out_f32, a.bias, a.out_stride, a.out_off, a.relu, a.accumulate, a.mask, a.m_stride,
+                  a.m_off, a.first_only};
     const int n_tile = tc_n_tile(a.Cout, tiles, sms);
     constexpr CUtensorMapSwizzle sw = KC == 16 ? CU_TENSOR_MAP_SWIZZLE_32B
                                     : (KC == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B);
@@ -1473,7 +1493,8 @@ cudaError_t slab_launch(const ConvArgs &a, const SlabPlan &p, int sms, cudaStrea
     t.by = p.by; t.bz = p.bz; t.g = 128 / a.W; t.gyn = p.gyn; t.n_acc = p.n_acc;
     t.tiles_y = (a.H + p.by - 1) / p.by;
     t.tiles_z = (a.D + p.bz - 1) / p.bz;
-    t.o = ConvOut{a.out, a.out_f32, a.bias, a.out_stride, a.out_off, a.relu, a.accumulate};
+    t.o = ConvOut{a.out, a.out_f32, a.bias, a.out_stride, a.out_off, a.relu, a.accumulate, a.mask, a.m_stride,
+                  a.m_off, a.first_only};
     constexpr CUtensorMapSwizzle sw = KC == 16 ? CU_TENSOR_MAP_SWIZZLE_32B
                                     : (KC == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B);
     CUtensorMap map_in, map_w;
@@ -1731,40 +1752,69 @@ struct Buf {
     void release() { if (p) cudaFree(p); p = nullptr; n = 0; }
 };
 
+// Offset of layer l's weights in the packed parameter vector (its biases
+// follow them): multiples of 16, so that every tensor starts 32-byte aligned.
+constexpr long long weight_off(int l)
+{
+    long long o = 0;
+    for (int k = 0; k < l; ++k) o += (long long)kSpec[k].cout * 27 * kSpec[k].cin + kSpec[k].cout;
+    return o;
+}
+constexpr long long bias_off(int l) { return weight_off(l) + (long long)kSpec[l].cout * 27 * kSpec[l].cin; }
+constexpr long long kParams = weight_off(kLayers);
+
+struct LayerOffsets { long long w[kLayers]; int cin[kLayers], cout[kLayers]; };
+constexpr LayerOffsets layer_offsets()
+{
+    LayerOffsets t{};
+    for (int l = 0; l < kLayers; ++l) { t.w[l] = weight_off(l); t.cin[l] = kSpec[l].cin; t.cout[l] = kSpec[l].cout; }
+    return t;
+}
+__constant__ const LayerOffsets c_layers = layer_offsets();
+
+// The transposed convolutions' weights of every layer but the first (whose
+// input gradient nobody needs), blockIdx.y = layer - 1: one launch instead of
+// one per layer.
+__global__ void flip_all_weights_kernel(const bf16 *W, bf16 *Wt)
+{
+    const int l = blockIdx.y + 1;
+    flip_weights<unsigned>(W + c_layers.w[l], c_layers.cout[l], c_layers.cin[l], Wt + c_layers.w[l]);
+}
+
 struct Net {
     int device = 0;
     int batch = 0, S = 0, n_in = 2;              // n_in: real input channels (of the 16)
     long long V0 = 0, V1 = 0, V2 = 0, V3 = 0;     // voxels per level (all samples)
-    // parameters
-    Buf<float> w32[kLayers], b32[kLayers], gw[kLayers], gb[kLayers], mw[kLayers], vw[kLayers], mb[kLayers], vb[kLayers];
-    Buf<bf16> w16[kLayers], wt[kLayers];
+    // parameters, gradients and Adam moments, packed as soc_unet_set_params
+    // has them (one copy, clear or update is one launch); BF16 weights and
+    // flipped weights at the same offsets
+    Buf<float> par, grad, mom, var;
+    Buf<bf16> par16, wt;
     long long adam_t = 0;
     // activations (BF16)
     Buf<bf16> x16, e0a, cat0, p0, e1a, cat1, p1, e2a, cat2, p2, b_a, b_b, d2a, d2b, d1a, d1b, d0a, d0b;
     Buf<uint8_t> arg0, arg1, arg2;
-    Buf<float> head;
-    // gradients (FP32) and a BF16 staging buffer
-    Buf<float> g_head, g_d0b, g_d0a, g_cat0, g_d1b, g_d1a, g_cat1, g_d2b, g_d2a, g_cat2, g_bb, g_ba, g_p2, g_e2a, g_p1,
-        g_e1a, g_p0, g_e0a;
-    Buf<bf16> gstage;
+    Buf<float> head;              // the prediction
+    // gradients: FP32 where a second kernel adds to them, else BF16, masked,
+    // in two buffers used in turn
+    Buf<float> g_cat0, g_cat1, g_cat2, g_p2, g_p1, g_p0;
+    Buf<bf16> g16[2];
     Buf<double> loss, loss_part;
     Buf<float> part;              // per-block partial sums of the weight and bias gradients
+
+    float *bias(int l) { return par.p + bias_off(l); }
+    bf16 *w16(int l) { return par16.p + weight_off(l); }
 
     template <class F>
     void each(F f)
     {
-        for (int l = 0; l < kLayers; ++l) {
-            f(w32[l]); f(b32[l]); f(gw[l]); f(gb[l]); f(mw[l]); f(vw[l]); f(mb[l]); f(vb[l]);
-        }
-        f(head); f(g_head); f(g_d0b); f(g_d0a); f(g_cat0); f(g_d1b); f(g_d1a); f(g_cat1); f(g_d2b); f(g_d2a);
-        f(g_cat2); f(g_bb); f(g_ba); f(g_p2); f(g_e2a); f(g_p1); f(g_e1a); f(g_p0); f(g_e0a); f(part);
+        f(par); f(grad); f(mom); f(var); f(head); f(g_cat0); f(g_cat1); f(g_cat2); f(g_p2); f(g_p1); f(g_p0); f(part);
     }
     template <class F>
     void each16(F f)
     {
-        for (int l = 0; l < kLayers; ++l) { f(w16[l]); f(wt[l]); }
-        f(x16); f(e0a); f(cat0); f(p0); f(e1a); f(cat1); f(p1); f(e2a); f(cat2); f(p2); f(b_a); f(b_b); f(d2a);
-        f(d2b); f(d1a); f(d1b); f(d0a); f(d0b); f(gstage);
+        f(par16); f(wt); f(x16); f(e0a); f(cat0); f(p0); f(e1a); f(cat1); f(p1); f(e2a); f(cat2); f(p2); f(b_a); f(b_b);
+        f(d2a); f(d2b); f(d1a); f(d1b); f(d0a); f(d0b); f(g16[0]); f(g16[1]);
     }
     void release()
     {
@@ -1838,39 +1888,44 @@ ConvArgs conv_args(const bf16 *in, int in_stride, int in_off, const bf16 *w, con
 soc_status fwd(Net &n, int l, const bf16 *in, int in_stride, int in_off, int S, bf16 *out, int out_stride, int out_off,
                cudaStream_t s)
 {
-    ConvArgs a = conv_args(in, in_stride, in_off, n.w16[l].p, n.b32[l].p, n.batch, S, kSpec[l].cin, kSpec[l].cout,
+    ConvArgs a = conv_args(in, in_stride, in_off, n.w16(l), n.bias(l), n.batch, S, kSpec[l].cin, kSpec[l].cout,
                            kSpec[l].relu);
     a.out = out; a.out_stride = out_stride; a.out_off = out_off;
     NNCK(conv_launch(a, s));
     return SOC_OK;
 }
 
-// backward of one layer: gy (FP32 view, masked by the layer's output y when it
-// has a ReLU) -> gw, gb, and (if gx) gx (FP32 view, accumulate or overwrite)
-soc_status bwd(Net &n, int l, const float *gy, int gy_stride, int gy_off, const bf16 *y, int y_stride, int y_off,
-               const bf16 *x, int x_stride, int x_off, int S, float *gx, int gx_stride, int gx_off, int accumulate,
-               cudaStream_t s)
+// Where a layer's input gradient goes: a dense FP32 tensor, or BF16 (dense)
+// masked by the ReLU of the layer below, whose output `mask` is (dense).
+struct GradOut {
+    float *f32 = nullptr;
+    bf16 *b16 = nullptr;
+    const bf16 *mask = nullptr;
+};
+
+// backward of one layer: gy (dense BF16, masked by the layer's own ReLU) ->
+// gw, gb and the input gradient
+soc_status bwd(Net &n, int l, const bf16 *gy, const bf16 *x, int S, const GradOut &g, cudaStream_t s)
 {
     const int Cin = kSpec[l].cin, Cout = kSpec[l].cout;
     const long long V = (long long)n.batch * S * S * S;
-    mask_to_bf16_kernel<<<grid_all(V), 256, 0, s>>>(gy, gy_stride, gy_off, kSpec[l].relu ? y : nullptr, y_stride,
-                                                         y_off, Cout, V, n.gstage.p);
-    NNCK(cudaGetLastError());
     WgradArgs wa;
     memset(&wa, 0, sizeof wa);
-    wa.gy = n.gstage.p; wa.gy_stride = Cout; wa.gy_off = 0; wa.x = x; wa.x_stride = x_stride; wa.x_off = x_off;
+    wa.gy = gy; wa.gy_stride = Cout; wa.x = x; wa.x_stride = Cin;
     wa.part = n.part.p; wa.N = n.batch; wa.D = S; wa.H = S; wa.W = S; wa.Cin = Cin; wa.Cout = Cout;
-    NNCK(wgrad_launch(wa, n.gw[l].p, (long long)n.part.n, s));
-    NNCK(bias_grad_launch(n.gstage.p, Cout, V, n.gb[l].p, n.part.p, (long long)n.part.n, s));
-    if (gx) {
-        ConvArgs a = conv_args(n.gstage.p, Cout, 0, n.wt[l].p, nullptr, n.batch, S, Cout, Cin, 0);
-        a.out_f32 = gx; a.out_stride = gx_stride; a.out_off = gx_off; a.accumulate = accumulate;
+    NNCK(wgrad_launch(wa, n.grad.p + weight_off(l), (long long)n.part.n, s));
+    NNCK(bias_grad_launch(gy, Cout, V, n.grad.p + bias_off(l), n.part.p, (long long)n.part.n, s));
+    if (g.f32 || g.b16) {
+        ConvArgs a = conv_args(gy, Cout, 0, n.wt.p + weight_off(l), nullptr, n.batch, S, Cout, Cin, 0);
+        a.out_f32 = g.f32; a.out = g.b16; a.out_stride = Cin;
+        a.mask = g.mask; a.m_stride = Cin;
         NNCK(conv_launch(a, s));
     }
     return SOC_OK;
 }
 
-soc_status forward(Net &n, const float *d_in, cudaStream_t s)
+// the network's prediction into pred [V0]
+soc_status forward(Net &n, const float *d_in, float *pred, cudaStream_t s)
 {
     const int S0 = n.S, S1 = S0 / 2, S2 = S0 / 4, S3 = S0 / 8;
     soc_status st;
@@ -1896,53 +1951,57 @@ soc_status forward(Net &n, const float *d_in, cudaStream_t s)
     upsample_kernel<<<grid_rows(S0 * 4, (long long)n.batch * S0 * S0), 128, 0, s>>>(n.d1b.p, n.batch, S1, S1, S1, 32, n.cat0.p, 48, 0);
     if ((st = fwd(n, 12, n.cat0.p, 48, 0, S0, n.d0a.p, 16, 0, s))) return st;
     if ((st = fwd(n, 13, n.d0a.p, 16, 0, S0, n.d0b.p, 16, 0, s))) return st;
-    ConvArgs a = conv_args(n.d0b.p, 16, 0, n.w16[14].p, n.b32[14].p, n.batch, S0, 16, 16, 0);
-    a.out_f32 = n.head.p; a.out_stride = 16; a.out_off = 0;
+    ConvArgs a = conv_args(n.d0b.p, 16, 0, n.w16(14), n.bias(14), n.batch, S0, 16, 16, 0);
+    a.out_f32 = pred; a.out_stride = 16; a.first_only = 1;
     NNCK(conv_launch(a, s));
     return SOC_OK;
 }
 
-soc_status backward(Net &n, const float *d_target, cudaStream_t s)
+// gradients of the loss at the prediction `pred`
+soc_status backward(Net &n, const float *pred, const float *d_target, cudaStream_t s)
 {
-    const int S0 = n.S, S1 = S0 / 2, S2 = S0 / 4, S3 = S0 / 8;
+    const int S0 = n.S, S1 = S0 / 2, S2 = S0 / 4, S3 = S0 / 8, B = n.batch;
     soc_status st;
-    for (int l = 0; l < kLayers; ++l) {
-        NNCK(cudaMemsetAsync(n.gw[l].p, 0, n.gw[l].n * 4, s));
-        NNCK(cudaMemsetAsync(n.gb[l].p, 0, n.gb[l].n * 4, s));
-        flip_weights_kernel<<<grid_1d((long long)kSpec[l].cout * 27 * kSpec[l].cin), 256, 0, s>>>(
-            n.w16[l].p, kSpec[l].cout, kSpec[l].cin, n.wt[l].p);
-    }
-    NNCK(cudaMemsetAsync(n.g_head.p, 0, n.g_head.n * 4, s));
-    mse_kernel<<<grid_1d(n.V0), 256, 0, s>>>(n.head.p, d_target, n.V0, nullptr, n.g_head.p, n.loss_part.p);
+    bf16 *const ga = n.g16[0].p, *const gb = n.g16[1].p;
+    auto masked = [](bf16 *out, const bf16 *mask) { GradOut g; g.b16 = out; g.mask = mask; return g; };
+    auto plain = [](float *out) { GradOut g; g.f32 = out; return g; };
+    NNCK(cudaMemsetAsync(n.grad.p, 0, sizeof(float) * n.grad.n, s));
+    flip_all_weights_kernel<<<dim3(48, kLayers - 1), 256, 0, s>>>(n.par16.p, n.wt.p);
+    mse_kernel<<<grid_1d(n.V0), 256, 0, s>>>(pred, d_target, n.V0, ga, n.loss_part.p);
     sum_loss_kernel<<<1, 256, 0, s>>>(n.loss_part.p, grid_1d(n.V0), n.loss.p);
     NNCK(cudaGetLastError());
     // decoder level 0
-    if ((st = bwd(n, 14, n.g_head.p, 16, 0, nullptr, 0, 0, n.d0b.p, 16, 0, S0, n.g_d0b.p, 16, 0, 0, s))) return st;
-    if ((st = bwd(n, 13, n.g_d0b.p, 16, 0, n.d0b.p, 16, 0, n.d0a.p, 16, 0, S0, n.g_d0a.p, 16, 0, 0, s))) return st;
-    if ((st = bwd(n, 12, n.g_d0a.p, 16, 0, n.d0a.p, 16, 0, n.cat0.p, 48, 0, S0, n.g_cat0.p, 48, 0, 0, s))) return st;
-    upsample_bwd_kernel<<<grid_rows(S1 * 8, (long long)n.batch * S1 * S1), 128, 0, s>>>(n.g_cat0.p, 48, 0, n.batch, S1, S1, S1, 32, n.g_d1b.p);
+    if ((st = bwd(n, 14, ga, n.d0b.p, S0, masked(gb, n.d0b.p), s))) return st;
+    if ((st = bwd(n, 13, gb, n.d0a.p, S0, masked(ga, n.d0a.p), s))) return st;
+    if ((st = bwd(n, 12, ga, n.cat0.p, S0, plain(n.g_cat0.p), s))) return st;
+    upsample_bwd_kernel<<<grid_rows(S1 * 4, (long long)B * S1 * S1), 128, 0, s>>>(n.g_cat0.p, 48, 0, B, S1, S1, S1, 32,
+                                                                                  n.d1b.p, gb);
     // decoder level 1
-    if ((st = bwd(n, 11, n.g_d1b.p, 32, 0, n.d1b.p, 32, 0, n.d1a.p, 32, 0, S1, n.g_d1a.p, 32, 0, 0, s))) return st;
-    if ((st = bwd(n, 10, n.g_d1a.p, 32, 0, n.d1a.p, 32, 0, n.cat1.p, 96, 0, S1, n.g_cat1.p, 96, 0, 0, s))) return st;
-    upsample_bwd_kernel<<<grid_rows(S2 * 16, (long long)n.batch * S2 * S2), 128, 0, s>>>(n.g_cat1.p, 96, 0, n.batch, S2, S2, S2, 64, n.g_d2b.p);
+    if ((st = bwd(n, 11, gb, n.d1a.p, S1, masked(ga, n.d1a.p), s))) return st;
+    if ((st = bwd(n, 10, ga, n.cat1.p, S1, plain(n.g_cat1.p), s))) return st;
+    upsample_bwd_kernel<<<grid_rows(S2 * 8, (long long)B * S2 * S2), 128, 0, s>>>(n.g_cat1.p, 96, 0, B, S2, S2, S2, 64,
+                                                                                  n.d2b.p, gb);
     // decoder level 2
-    if ((st = bwd(n, 9, n.g_d2b.p, 64, 0, n.d2b.p, 64, 0, n.d2a.p, 64, 0, S2, n.g_d2a.p, 64, 0, 0, s))) return st;
-    if ((st = bwd(n, 8, n.g_d2a.p, 64, 0, n.d2a.p, 64, 0, n.cat2.p, 192, 0, S2, n.g_cat2.p, 192, 0, 0, s))) return st;
-    upsample_bwd_kernel<<<grid_rows(S3 * 32, (long long)n.batch * S3 * S3), 128, 0, s>>>(n.g_cat2.p, 192, 0, n.batch, S3, S3, S3, 128, n.g_bb.p);
+    if ((st = bwd(n, 9, gb, n.d2a.p, S2, masked(ga, n.d2a.p), s))) return st;
+    if ((st = bwd(n, 8, ga, n.cat2.p, S2, plain(n.g_cat2.p), s))) return st;
+    upsample_bwd_kernel<<<grid_rows(S3 * 16, (long long)B * S3 * S3), 128, 0, s>>>(n.g_cat2.p, 192, 0, B, S3, S3, S3, 128,
+                                                                                   n.b_b.p, gb);
     // bottleneck
-    if ((st = bwd(n, 7, n.g_bb.p, 128, 0, n.b_b.p, 128, 0, n.b_a.p, 128, 0, S3, n.g_ba.p, 128, 0, 0, s))) return st;
-    if ((st = bwd(n, 6, n.g_ba.p, 128, 0, n.b_a.p, 128, 0, n.p2.p, 64, 0, S3, n.g_p2.p, 64, 0, 0, s))) return st;
-    maxpool_bwd_kernel<<<grid_rows(S3 * 8, (long long)n.batch * S3 * S3), 128, 0, s>>>(n.g_p2.p, n.arg2.p, n.batch, S2, S2, S2, 64, n.g_cat2.p, 192,
-                                                          128);
+    if ((st = bwd(n, 7, gb, n.b_a.p, S3, masked(ga, n.b_a.p), s))) return st;
+    if ((st = bwd(n, 6, ga, n.p2.p, S3, plain(n.g_p2.p), s))) return st;
     // encoder level 2 (its output is the skip slice of cat2)
-    if ((st = bwd(n, 5, n.g_cat2.p, 192, 128, n.cat2.p, 192, 128, n.e2a.p, 64, 0, S2, n.g_e2a.p, 64, 0, 0, s))) return st;
-    if ((st = bwd(n, 4, n.g_e2a.p, 64, 0, n.e2a.p, 64, 0, n.p1.p, 32, 0, S2, n.g_p1.p, 32, 0, 0, s))) return st;
-    maxpool_bwd_kernel<<<grid_rows(S2 * 4, (long long)n.batch * S2 * S2), 128, 0, s>>>(n.g_p1.p, n.arg1.p, n.batch, S1, S1, S1, 32, n.g_cat1.p, 96, 64);
-    if ((st = bwd(n, 3, n.g_cat1.p, 96, 64, n.cat1.p, 96, 64, n.e1a.p, 32, 0, S1, n.g_e1a.p, 32, 0, 0, s))) return st;
-    if ((st = bwd(n, 2, n.g_e1a.p, 32, 0, n.e1a.p, 32, 0, n.p0.p, 16, 0, S1, n.g_p0.p, 16, 0, 0, s))) return st;
-    maxpool_bwd_kernel<<<grid_rows(S1 * 2, (long long)n.batch * S1 * S1), 128, 0, s>>>(n.g_p0.p, n.arg0.p, n.batch, S0, S0, S0, 16, n.g_cat0.p, 48, 32);
-    if ((st = bwd(n, 1, n.g_cat0.p, 48, 32, n.cat0.p, 48, 32, n.e0a.p, 16, 0, S0, n.g_e0a.p, 16, 0, 0, s))) return st;
-    if ((st = bwd(n, 0, n.g_e0a.p, 16, 0, n.e0a.p, 16, 0, n.x16.p, 16, 0, S0, nullptr, 0, 0, 0, s))) return st;
+    maxpool_bwd_kernel<<<grid_rows(S3 * 8, (long long)B * S3 * S3), 128, 0, s>>>(
+        n.g_p2.p, n.arg2.p, B, S2, S2, S2, 64, n.g_cat2.p, 192, 128, n.cat2.p, 192, 128, gb);
+    if ((st = bwd(n, 5, gb, n.e2a.p, S2, masked(ga, n.e2a.p), s))) return st;
+    if ((st = bwd(n, 4, ga, n.p1.p, S2, plain(n.g_p1.p), s))) return st;
+    maxpool_bwd_kernel<<<grid_rows(S2 * 4, (long long)B * S2 * S2), 128, 0, s>>>(
+        n.g_p1.p, n.arg1.p, B, S1, S1, S1, 32, n.g_cat1.p, 96, 64, n.cat1.p, 96, 64, gb);
+    if ((st = bwd(n, 3, gb, n.e1a.p, S1, masked(ga, n.e1a.p), s))) return st;
+    if ((st = bwd(n, 2, ga, n.p0.p, S1, plain(n.g_p0.p), s))) return st;
+    maxpool_bwd_kernel<<<grid_rows(S1 * 2, (long long)B * S1 * S1), 128, 0, s>>>(
+        n.g_p0.p, n.arg0.p, B, S0, S0, S0, 16, n.g_cat0.p, 48, 32, n.cat0.p, 48, 32, gb);
+    if ((st = bwd(n, 1, gb, n.e0a.p, S0, masked(ga, n.e0a.p), s))) return st;
+    if ((st = bwd(n, 0, ga, n.x16.p, S0, GradOut{}, s))) return st;
     NNCK(cudaGetLastError());
     return SOC_OK;
 }
@@ -1965,22 +2024,16 @@ soc_status soc_unet_create(int device, int batch, int side, int n_inputs, int *n
     n->V1 = n->V0 / 8; n->V2 = n->V1 / 8; n->V3 = n->V2 / 8;
     cudaError_t e = cudaSuccess;
     auto A = [&](auto &b, size_t cnt) { if (e == cudaSuccess) e = b.alloc(cnt); };
-    for (int l = 0; l < kLayers; ++l) {
-        const size_t nw = (size_t)kSpec[l].cout * 27 * kSpec[l].cin, nb = kSpec[l].cout;
-        A(n->w32[l], nw); A(n->gw[l], nw); A(n->mw[l], nw); A(n->vw[l], nw); A(n->w16[l], nw); A(n->wt[l], nw);
-        A(n->b32[l], nb); A(n->gb[l], nb); A(n->mb[l], nb); A(n->vb[l], nb);
-    }
+    A(n->par, kParams); A(n->grad, kParams); A(n->mom, kParams); A(n->var, kParams); A(n->par16, kParams); A(n->wt, kParams);
     A(n->x16, n->V0 * 16); A(n->e0a, n->V0 * 16); A(n->cat0, n->V0 * 48); A(n->p0, n->V1 * 16);
     A(n->e1a, n->V1 * 32); A(n->cat1, n->V1 * 96); A(n->p1, n->V2 * 32); A(n->e2a, n->V2 * 64);
     A(n->cat2, n->V2 * 192); A(n->p2, n->V3 * 64); A(n->b_a, n->V3 * 128); A(n->b_b, n->V3 * 128);
     A(n->d2a, n->V2 * 64); A(n->d2b, n->V2 * 64); A(n->d1a, n->V1 * 32); A(n->d1b, n->V1 * 32);
-    A(n->d0a, n->V0 * 16); A(n->d0b, n->V0 * 16); A(n->head, n->V0 * 16);
+    A(n->d0a, n->V0 * 16); A(n->d0b, n->V0 * 16); A(n->head, n->V0);
     A(n->arg0, n->V1 * 16); A(n->arg1, n->V2 * 32); A(n->arg2, n->V3 * 64);
-    A(n->g_head, n->V0 * 16); A(n->g_d0b, n->V0 * 16); A(n->g_d0a, n->V0 * 16); A(n->g_cat0, n->V0 * 48);
-    A(n->g_d1b, n->V1 * 32); A(n->g_d1a, n->V1 * 32); A(n->g_cat1, n->V1 * 96); A(n->g_d2b, n->V2 * 64);
-    A(n->g_d2a, n->V2 * 64); A(n->g_cat2, n->V2 * 192); A(n->g_bb, n->V3 * 128); A(n->g_ba, n->V3 * 128);
-    A(n->g_p2, n->V3 * 64); A(n->g_e2a, n->V2 * 64); A(n->g_p1, n->V2 * 32); A(n->g_e1a, n->V1 * 32);
-    A(n->g_p0, n->V1 * 16); A(n->g_e0a, n->V0 * 16); A(n->gstage, n->V0 * 48); A(n->loss, 1);
+    A(n->g_cat0, n->V0 * 48); A(n->g_cat1, n->V1 * 96); A(n->g_cat2, n->V2 * 192);
+    A(n->g_p2, n->V3 * 64); A(n->g_p1, n->V2 * 32); A(n->g_p0, n->V1 * 16);
+    A(n->g16[0], n->V0 * 16); A(n->g16[1], n->V0 * 16); A(n->loss, 1);
     A(n->loss_part, (size_t)grid_1d(n->V0));
     {   // partial sums: the largest weight (or bias) gradient of any layer
         long long need = 0;
@@ -1993,12 +2046,10 @@ soc_status soc_unet_create(int device, int batch, int side, int n_inputs, int *n
         A(n->part, (size_t)need);
     }
     if (e != cudaSuccess) { n->release(); delete n; return SOC_ERR_NOMEM; }
-    for (int l = 0; l < kLayers; ++l) {
-        cudaMemset(n->mw[l].p, 0, n->mw[l].n * 4); cudaMemset(n->vw[l].p, 0, n->vw[l].n * 4);
-        cudaMemset(n->mb[l].p, 0, n->mb[l].n * 4); cudaMemset(n->vb[l].p, 0, n->vb[l].n * 4);
-        cudaMemset(n->w32[l].p, 0, n->w32[l].n * 4); cudaMemset(n->b32[l].p, 0, n->b32[l].n * 4);
-        cudaMemset(n->w16[l].p, 0, n->w16[l].n * 2);
-    }
+    cudaMemset(n->par.p, 0, sizeof(float) * kParams);
+    cudaMemset(n->mom.p, 0, sizeof(float) * kParams);
+    cudaMemset(n->var.p, 0, sizeof(float) * kParams);
+    cudaMemset(n->par16.p, 0, sizeof(bf16) * kParams);
     try {                                  // no exception crosses the C ABI
         std::lock_guard<std::mutex> lock(g_nets.m);
         g_nets.nets.push_back(n);
@@ -2025,26 +2076,15 @@ soc_status soc_unet_destroy(int net_id)
     return SOC_OK;
 }
 
-int64_t soc_unet_param_count(void)
-{
-    int64_t c = 0;
-    for (int l = 0; l < kLayers; ++l) c += (int64_t)kSpec[l].cout * 27 * kSpec[l].cin + kSpec[l].cout;
-    return c;
-}
+int64_t soc_unet_param_count(void) { return kParams; }
 
 soc_status soc_unet_set_params(int net_id, const float *host)
 {
     Net *n = net_of(net_id);
     if (!n || !host) return SOC_ERR_ARG;
-    const float *p = host;
-    for (int l = 0; l < kLayers; ++l) {
-        NNCK(cudaMemcpy(n->w32[l].p, p, n->w32[l].n * 4, cudaMemcpyHostToDevice));
-        p += n->w32[l].n;
-        NNCK(cudaMemcpy(n->b32[l].p, p, n->b32[l].n * 4, cudaMemcpyHostToDevice));
-        p += n->b32[l].n;
-        to_bf16_kernel<<<grid_1d((long long)n->w32[l].n), 256>>>(n->w32[l].p, (long long)n->w32[l].n, n->w16[l].p);
-        NNCK(cudaGetLastError());
-    }
+    NNCK(cudaMemcpy(n->par.p, host, sizeof(float) * kParams, cudaMemcpyHostToDevice));
+    to_bf16_kernel<<<grid_1d(kParams), 256>>>(n->par.p, kParams, n->par16.p);
+    NNCK(cudaGetLastError());
     NNCK(cudaDeviceSynchronize());
     n->adam_t = 0;
     return SOC_OK;
@@ -2055,13 +2095,7 @@ soc_status soc_unet_get_params(int net_id, float *host, int grads)
     Net *n = net_of(net_id);
     if (!n || !host) return SOC_ERR_ARG;
     NNCK(cudaDeviceSynchronize());
-    float *p = host;
-    for (int l = 0; l < kLayers; ++l) {
-        NNCK(cudaMemcpy(p, grads ? n->gw[l].p : n->w32[l].p, n->w32[l].n * 4, cudaMemcpyDeviceToHost));
-        p += n->w32[l].n;
-        NNCK(cudaMemcpy(p, grads ? n->gb[l].p : n->b32[l].p, n->b32[l].n * 4, cudaMemcpyDeviceToHost));
-        p += n->b32[l].n;
-    }
+    NNCK(cudaMemcpy(host, grads ? n->grad.p : n->par.p, sizeof(float) * kParams, cudaMemcpyDeviceToHost));
     return SOC_OK;
 }
 
@@ -2070,11 +2104,7 @@ soc_status soc_unet_forward(int net_id, const float *d_input, float *d_pred, voi
     Net *n = net_of(net_id);
     if (!n || !d_input || !d_pred) return SOC_ERR_ARG;
     cudaStream_t s = (cudaStream_t)stream;
-    soc_status st = forward(*n, d_input, s);
-    if (st) return st;
-    mse_kernel<<<grid_1d(n->V0), 256, 0, s>>>(n->head.p, nullptr, n->V0, d_pred, nullptr, nullptr);
-    NNCK(cudaGetLastError());
-    return SOC_OK;
+    return forward(*n, d_input, d_pred, s);
 }
 
 soc_status soc_unet_backward(int net_id, const float *d_input, const float *d_target, float *d_pred, double *d_loss,
@@ -2083,13 +2113,10 @@ soc_status soc_unet_backward(int net_id, const float *d_input, const float *d_ta
     Net *n = net_of(net_id);
     if (!n || !d_input || !d_target) return SOC_ERR_ARG;
     cudaStream_t s = (cudaStream_t)stream;
-    soc_status st = forward(*n, d_input, s);
+    float *const pred = d_pred ? d_pred : n->head.p;
+    soc_status st = forward(*n, d_input, pred, s);
     if (st) return st;
-    if (d_pred) {
-        mse_kernel<<<grid_1d(n->V0), 256, 0, s>>>(n->head.p, nullptr, n->V0, d_pred, nullptr, nullptr);
-        NNCK(cudaGetLastError());
-    }
-    if ((st = backward(*n, d_target, s))) return st;
+    if ((st = backward(*n, pred, d_target, s))) return st;
     if (d_loss) NNCK(cudaMemcpyAsync(d_loss, n->loss.p, 8, cudaMemcpyDeviceToDevice, s));
     return SOC_OK;
 }
@@ -2105,14 +2132,8 @@ soc_status soc_unet_adam(int net_id, float lr, void *stream)
     // 7e-6 relative error at t = 2), then rounded once
     const float c1 = (float)(1.0 - std::pow((double)b1, (double)n->adam_t));
     const float c2 = (float)(1.0 - std::pow((double)b2, (double)n->adam_t));
-    for (int l = 0; l < kLayers; ++l) {
-        adam_kernel<<<grid_1d((long long)n->w32[l].n), 256, 0, s>>>(n->w32[l].p, n->mw[l].p, n->vw[l].p, n->gw[l].p,
-                                                                   (long long)n->w32[l].n, lr, b1, b2, eps, c1, c2,
-                                                                   n->w16[l].p);
-        adam_kernel<<<grid_1d((long long)n->b32[l].n), 256, 0, s>>>(n->b32[l].p, n->mb[l].p, n->vb[l].p, n->gb[l].p,
-                                                                   (long long)n->b32[l].n, lr, b1, b2, eps, c1, c2,
-                                                                   nullptr);
-    }
+    adam_kernel<<<grid_1d(kParams), 256, 0, s>>>(n->par.p, n->mom.p, n->var.p, n->grad.p, kParams, lr, b1, b2, eps, c1,
+                                                 c2, n->par16.p);
     NNCK(cudaGetLastError());
     return SOC_OK;
 }
