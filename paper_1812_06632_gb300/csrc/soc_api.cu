@@ -108,7 +108,7 @@ struct soc_ctx {
     DevBuf<unsigned long long> d_wscratch;
     DevBuf<double> d_maxdT;
     DevBuf<int64_t> d_level_start;
-    DevBuf<double> d_map_S;       // per-cell source function of the last map
+    DevBuf<float2> d_map_S;       // per-cell source function of the last map
     // pinned staging of grid uploads (grows to the largest grid)
     uint32_t *h_stage = nullptr;
     size_t h_stage_n = 0;
@@ -1374,9 +1374,16 @@ soc_status soc_map(soc_ctx *ctx, int cloud_id, const float *d_T, int freq, const
         M.npx = npx;
         M.npy = npy;
         M.max_cells = 100000000u;
+        const double c2 = 1.4426950408889634 * (kHc * M.nu / kKc);
+        M.src_c = make_float2((float)c2, (float)(c2 - (double)(float)c2));
+        const double r = M.kabs_over_kext * (2.0 * kHc * M.nu * M.nu * M.nu / (kCc * kCc));
+        int re = 0;
+        const double rm = 2.0 * std::frexp(r, &re);               // r = rm 2^(re - 1), rm in [1, 2), or 0
+        M.src_r = make_float2((float)rm, (float)(rm - (double)(float)rm));
+        M.src_e = r > 0.0 && std::isfinite(r) ? re - 1 + 64 : 1000;
         CK(ctx->d_map_S.alloc(cl.n_cells), "map source scratch");
         M.S = ctx->d_map_S.p;
-        CK(launch_map(M, cl.n_cells, ctx->sms, (cudaStream_t)stream), "map");
+        CK(launch_map(M, cl.n_cells, cl.n_levels == 1, ctx->sms, (cudaStream_t)stream), "map");
         return SOC_OK;
     });
 }

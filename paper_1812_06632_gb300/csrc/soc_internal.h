@@ -87,7 +87,9 @@ int trace_block_limit(int block, int variant, bool regular);   // max resident b
 struct MapParams {
     const DevCloud *cloud;
     const float *T;               // [n_cells]
-    double *S;                    // [n_cells] scratch: (kabs/kext) B_nu(T) per cell
+    float2 *S;                    // [n_cells] scratch: 2^64 (kabs/kext) B_nu(T) per cell, hi + lo
+    float2 src_c, src_r;          // log2(e) h nu / k, and the mantissa of 2^64 (kabs/kext) 2 h nu^3 / c^2: hi + lo
+    int32_t src_e;                // its exponent (far out of range: every cell in FP64)
     float *map;                   // [npy][npx]
     double d[3], e1[3], e2[3], c[3];
     double pix, nu, kext_root, kabs_over_kext, I_bg;
@@ -95,8 +97,9 @@ struct MapParams {
     uint32_t max_cells;
 };
 
-// source-function pass over the n_cells cells into m.S, then one thread per pixel
-cudaError_t launch_map(const MapParams &m, int64_t n_cells, int sms, cudaStream_t s);
+// source-function pass over the n_cells cells into m.S, then one thread per
+// pixel; regular: a one-level grid
+cudaError_t launch_map(const MapParams &m, int64_t n_cells, bool regular, int sms, cudaStream_t s);
 
 struct TempTables {
     int n_freq;

@@ -12,6 +12,7 @@
 #include <cstdint>
 #include <algorithm>
 #include "soc_internal.h"
+#include "soc_pair.cuh"
 
 namespace soc {
 namespace {
@@ -278,7 +279,6 @@ constexpr int32_t kSeZero = 1 << 20, kSeSlow = 1 << 21;
 
 __device__ __forceinline__ float lg2(float v) { float r; asm("lg2.approx.f32 %0, %1;" : "=f"(r) : "f"(v)); return r; }
 __device__ __forceinline__ float ex2(float v) { float r; asm("ex2.approx.f32 %0, %1;" : "=f"(r) : "f"(v)); return r; }
-__device__ __forceinline__ float rcp(float v) { float r; asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(v)); return r; }
 
 __device__ __forceinline__ int exponent_of(double v) { return (int)((__double_as_longlong(v) >> 52) & 0x7FF) - 1023; }
 __device__ __forceinline__ double mantissa_of(double v)
@@ -477,42 +477,11 @@ __global__ void __launch_bounds__(256) dust_max_kernel(const DevCloud *__restric
     }
 }
 
-// 2^(j/32) - 1 as hi + lo, j = 0 .. 31 (Taylor series of exp(j ln2 / 32)).
-struct Exp2Table { float h[32], l[32]; };
-constexpr Exp2Table make_exp2_table()
-{
-    Exp2Table t{};
-    for (int j = 0; j < 32; ++j) {
-        const double a = 0.69314718055994530942 * j / 32.0;
-        double term = 1.0, sum = 0.0;
-        for (int n = 1; n < 24; ++n) { term = term * a / n; sum += term; }
-        t.h[j] = (float)sum;
-        t.l[j] = (float)(sum - (double)t.h[j]);
-    }
-    return t;
-}
-__device__ const Exp2Table g_exp2_table = make_exp2_table();
-
 __device__ __noinline__ unsigned long long dust_weight_exact(const DevCloud &C, const TempTables &tt, const float *T,
                                                              int32_t cell, int f, double m)
 {
     const double L = dust_L(C, tt, T, cell, f);
     return (unsigned long long)rint(__dmul_rn(__ddiv_rn(L, m), kWUnit));
-}
-
-// A sum of FP32 numbers a + b = s + e exactly (Knuth's two-sum; the short
-// form needs |a| >= |b| or a = 0).
-__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
-{
-    s = __fadd_rn(a, b);
-    const float t = __fsub_rn(s, a);
-    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
-}
-__device__ __forceinline__ void quick_two_sum(float a, float b, float &s, float &e)
-{
-    const float t = __fadd_rn(a, b);
-    e = __fsub_rn(b, __fsub_rn(t, a));
-    s = t;
 }
 
 __global__ void __launch_bounds__(256) dust_weight_kernel(const DevCloud *__restrict__ dcl, int64_t n_leaf,
@@ -531,7 +500,6 @@ __global__ void __launch_bounds__(256) dust_weight_kernel(const DevCloud *__rest
         e_unit[f0 + threadIdx.x] = __ddiv_rn(__ddiv_rn(m, (double)n_per_cell), kWUnit);
     }
     const DevCloud &C = *dcl;
-    constexpr float kLn2H = 0x1.62e43p-1f, kLn2L = -0x1.05c61p-29f;          // ln 2, hi + lo
     constexpr float k4PiH = 0x1.921fb6p+3f, k4PiL = -0x1.777a5cp-22f;        // 4 pi, hi + lo
     for (int64_t b = blockIdx.x * (int64_t)256; b < n_leaf; b += (int64_t)gridDim.x * 256) {
         const int64_t li = b + threadIdx.x;
@@ -553,11 +521,11 @@ __global__ void __launch_bounds__(256) dust_weight_kernel(const DevCloud *__rest
         const float gl = __fmaf_rn(r4l, vh, __fmaf_rn(r4h, vl, __fmaf_rn(r4h, vh, -gh)));
         for (int f = 0; f < nf; ++f) {
             const DustFreq F = s_f[f];
-            // y = log2(e) h nu / (k T) = n / 32 + s, |s| <= 1/64
+            // y = log2(e) h nu / (k T)
             const float p = __fmul_rn(F.ch, ih);
             const float pe = __fmaf_rn(F.cl, ih, __fmaf_rn(F.ch, il, __fmaf_rn(F.ch, ih, -p)));
-            const float tn = __fmaf_rn(fminf(p, 2048.0f), 32.0f, 12582912.0f);
-            const int n = __float_as_int(tn) - 0x4B400000;
+            const float tn = pair_grid(p);
+            const int n = pair_index(tn);
             const int k = n >> 5, e = ge + F.se - k;
             // W = 0: no density, an overflowing expm1 (y > 1024), a maximum
             // of 0, or v < 1/2 (the mantissas' quotient is below
@@ -569,34 +537,8 @@ __global__ void __launch_bounds__(256) dust_weight_kernel(const DevCloud *__rest
                 if (in) w[(int64_t)(f0 + f) * n_leaf + li] = 0;
                 continue;
             }
-            const float d = __fmaf_rn(__fsub_rn(tn, 12582912.0f), -0.03125f, p);
-            float sh, sl;
-            two_sum(d, pe, sh, sl);
-            // a = e^(s ln2) - 1 (Taylor to the fifth power)
-            const float rh = __fmul_rn(sh, kLn2H);
-            const float rl = __fmaf_rn(sl, kLn2H, __fmaf_rn(sh, kLn2L, __fmaf_rn(sh, kLn2H, -rh)));
-            const float r2 = __fmul_rn(rh, rh);
-            const float r2l = __fmaf_rn(__fadd_rn(rh, rh), rl, __fmaf_rn(rh, rh, -r2));
-            const float q = __fmul_rn(__fmul_rn(rh, r2), __fmaf_rn(rh, __fmaf_rn(rh, 0x1.111112p-7f, 0x1.555556p-5f),
-                                                                   0x1.555556p-3f));
-            float ah, al;
-            quick_two_sum(rh, __fmul_rn(0.5f, r2), ah, al);
-            al = __fadd_rn(al, __fadd_rn(__fmaf_rn(0.5f, r2l, rl), q));
-            // 2^(n/32 - k) e^(s ln2) - 1 = t + a + t a, t = 2^(j/32) - 1
-            const float t1 = __shfl_sync(0xffffffffu, th, n & 31), t1l = __shfl_sync(0xffffffffu, tl, n & 31);
-            const float ta = __fmul_rn(t1, ah);
-            const float tal = __fmaf_rn(t1l, ah, __fmaf_rn(t1, al, __fmaf_rn(t1, ah, -ta)));
-            float s1, e1, s2, e2;
-            quick_two_sum(t1, ah, s1, e1);
-            quick_two_sum(s1, ta, s2, e2);
-            const float lo = __fadd_rn(__fadd_rn(__fadd_rn(e1, e2), __fadd_rn(al, tal)), t1l);
-            // (e^x - 1) 2^-k = (1 - 2^-k) + that
-            const float mk = k < 120 ? __uint_as_float((uint32_t)(127 - max(k, 0)) << 23) : 0.0f;
-            const float c1 = __fsub_rn(1.0f, mk), ce = __fsub_rn(__fsub_rn(1.0f, c1), mk);
             float eh, el;
-            two_sum(c1, s2, eh, el);
-            // normalised: the quotient's correction is good to (el / eh)^2
-            quick_two_sum(eh, __fadd_rn(el, __fadd_rn(ce, lo)), eh, el);
+            pair_expm1(p, pe, tn, n, th, tl, eh, el);
             // v = g s / (e^x - 1)
             const float nh = __fmul_rn(gh, F.sh);
             const float nl = __fmaf_rn(gl, F.sh, __fmaf_rn(gh, F.sl, __fmaf_rn(gh, F.sh, -nh)));
