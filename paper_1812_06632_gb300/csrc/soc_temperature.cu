@@ -132,12 +132,38 @@ __device__ __forceinline__ void block_max_to(double v, unsigned long long *out)
     }
 }
 
+// Doubles as integers of the same order (no NaN): comparing these keeps the
+// twelve comparisons of a table search off the FP64 pipe (2.1e6 cells: 315 us,
+// 269 us with this; the logarithm and the exponential are the rest).
+__device__ __forceinline__ long long ordered_bits(double v)
+{
+    const long long b = __double_as_longlong(v);
+    return b ^ ((b >> 63) & 0x7FFFFFFFFFFFFFFFll);
+}
+
 // Equilibrium temperature: bracket ln A in the FP64 table of ln E(T_k) and
 // interpolate ln T linearly in ln E.  With 4096 log-spaced T_k the
 // interpolation error is below 2e-7 relative on the 64-frequency grid, far
 // inside the 1e-4 required against an FP64 root-finder, so no Newton step on
 // the quadrature is taken (it would cost 64 double-precision exponentials per
 // cell on a part whose FP64 rate is low).
+__device__ __forceinline__ double invert_table(const TempTables &tt, double a)
+{
+    if (!(a > 0.0)) return kTMin;
+    const double la = log(a);
+    if (la <= __ldg(tt.lnE)) return kTMin;
+    if (la >= __ldg(tt.lnE + kTableN - 1)) return kTMax;
+    const long long key = ordered_bits(la);
+    int lo = 0, hi = kTableN - 1;                             // lnE[lo] < la <= lnE[hi]
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (ordered_bits(__ldg(tt.lnE + mid)) < key) lo = mid; else hi = mid;
+    }
+    const double e0 = __ldg(tt.lnE + lo), e1 = __ldg(tt.lnE + hi);
+    const double t0 = __ldg(tt.lnT + lo), t1 = __ldg(tt.lnT + hi);
+    return fmin(fmax(exp(t0 + (la - e0) * (t1 - t0) / (e1 - e0)), kTMin), kTMax);
+}
+
 __global__ void temperature_kernel(const DevCloud *__restrict__ dcl, int64_t n_cells, const TempTables tt,
                                    const double *__restrict__ A, float *T, unsigned long long *max_dT)
 {
@@ -146,50 +172,11 @@ __global__ void temperature_kernel(const DevCloud *__restrict__ dcl, int64_t n_c
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < n_cells;
          c += (int64_t)gridDim.x * blockDim.x) {
         if (__ldg(C.cell + c) & kLinkBit) continue;                // refined cells carry no T
-        const double a = A[c];
-        double Tn;
-        if (!(a > 0.0)) {
-            Tn = kTMin;
-        } else {
-            const double la = log(a);
-            if (la <= __ldg(tt.lnE)) {
-                Tn = kTMin;
-            } else if (la >= __ldg(tt.lnE + kTableN - 1)) {
-                Tn = kTMax;
-            } else {
-                int lo = 0, hi = kTableN - 1;                         // lnE[lo] < la <= lnE[hi]
-                while (hi - lo > 1) {
-                    const int mid = (lo + hi) >> 1;
-                    if (__ldg(tt.lnE + mid) < la) lo = mid; else hi = mid;
-                }
-                const double e0 = __ldg(tt.lnE + lo), e1 = __ldg(tt.lnE + hi);
-                const double t0 = __ldg(tt.lnT + lo), t1 = __ldg(tt.lnT + hi);
-                Tn = exp(t0 + (la - e0) * (t1 - t0) / (e1 - e0));
-                Tn = fmin(fmax(Tn, kTMin), kTMax);
-            }
-        }
-        const float Tf = (float)Tn;
+        const float Tf = (float)invert_table(tt, A[c]);
         if (max_dT) dmax = fmax(dmax, fabs((double)Tf - (double)T[c]));
         T[c] = Tf;
     }
     if (max_dT) block_max_to(dmax, max_dT);
-}
-
-// T from A by the table (shared by both temperature kernels).
-__device__ __forceinline__ double invert_table(const TempTables &tt, double a)
-{
-    if (!(a > 0.0)) return kTMin;
-    const double la = log(a);
-    if (la <= __ldg(tt.lnE)) return kTMin;
-    if (la >= __ldg(tt.lnE + kTableN - 1)) return kTMax;
-    int lo = 0, hi = kTableN - 1;
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (__ldg(tt.lnE + mid) < la) lo = mid; else hi = mid;
-    }
-    const double e0 = __ldg(tt.lnE + lo), e1 = __ldg(tt.lnE + hi);
-    const double t0 = __ldg(tt.lnT + lo), t1 = __ldg(tt.lnT + hi);
-    return fmin(fmax(exp(t0 + (la - e0) * (t1 - t0) / (e1 - e0)), kTMin), kTMax);
 }
 
 // E(T) from the table (ln E linear in ln T between the log-spaced nodes).
@@ -259,7 +246,7 @@ __device__ __forceinline__ double dust_L(const DevCloud &C, const TempTables &tt
 //                      outside the ranges the bound covers, W is evaluated
 //                      in FP64 as above.
 // m, the weights and e_unit are therefore the FP64 evaluation's, bit for bit.
-// Measured on the same leaves: 0.13, 0.22 and 1.1 ms.
+// Measured on the same leaves: 0.13, 0.22 and 0.57 ms.
 // A thread takes leaves, a block kDustF frequencies (blockIdx.y) whose
 // constants it prepares in shared memory.
 // ---------------------------------------------------------------------------
@@ -271,8 +258,8 @@ constexpr float kInf = __builtin_huge_valf();
 struct DustFreq {
     float ch, cl;                        // log2(e) h nu / k (K), hi + lo
     float lf, lpre;                      // log2(kabs pre), log2(pre), pre = 2 h nu^3 / c^2; lpre = -inf: no bound
-    float sh, sl;                        // mantissa of kabs pre 2^31 / m, hi + lo (weights only)
-    int32_t se;                          // its exponent; kSeZero: m = 0, kSeSlow: no bound
+    float sh, sl;                        // mantissas' quotient of kabs pre 2^31 / m, hi + lo (weights only)
+    int32_t se;                          // the exponents' difference; kSeZero: m = 0, kSeSlow: no bound
     int32_t pad;
 };
 constexpr int32_t kSeZero = 1 << 20, kSeSlow = 1 << 21;
@@ -304,13 +291,13 @@ __device__ __forceinline__ DustFreq dust_freq(const TempTables &tt, int f, doubl
     if (weights) {
         if (m == 0.0) {
             d.se = kSeZero;
-        } else if (!ok || !(m > 0x1p-600 && m < 0x1p600)) {
+        } else if (!ok || !(m > 0x1p-1000 && m < 0x1p1000)) {
             d.se = kSeSlow;
         } else {
-            const double s = kp / m, sm = mantissa_of(s);
-            d.se = exponent_of(s) + 31;
-            d.sh = (float)sm;
-            d.sl = (float)(sm - (double)d.sh);
+            const double s = mantissa_of(kp) / mantissa_of(m);
+            d.se = exponent_of(kp) - exponent_of(m) + 31;
+            d.sh = (float)s;
+            d.sl = (float)(s - (double)d.sh);
         }
     }
     return d;
@@ -528,9 +515,9 @@ __global__ void __launch_bounds__(256) dust_weight_kernel(const DevCloud *__rest
             const int n = pair_index(tn);
             const int k = n >> 5, e = ge + F.se - k;
             // W = 0: no density, an overflowing expm1 (y > 1024), a maximum
-            // of 0, or v < 1/2 (the mantissas' quotient is below
-            // 4 / (2^2^-8 - 1) < 2^11); whole warps of such leaves are
-            // common where the maximum is a hot leaf's
+            // of 0, or v < 1/2 (the quotient of the mantissas is below
+            // 16 pi 2 / (2^2^-8 - 1) < 2^15.2); whole warps of such leaves
+            // are common where the maximum is a hot leaf's
             const bool plain = ok && F.se < kSeZero && p >= 0x1p-8f;
             const bool zero = !in || F.se == kSeZero || (plain && (rho == 0.0f || p > 1030.0f || e < -16));
             if (__all_sync(0xffffffffu, zero)) {
@@ -560,7 +547,8 @@ __global__ void __launch_bounds__(256) dust_weight_kernel(const DevCloud *__rest
                     // extended precision over x = 0.005 .. 600)
                     const float err = __fmaf_rn(vvh, __fmaf_rn(p, 0x1p-44f, __fmaf_rn(rc, 0x1p-42f, 0x1p-42f)), 0x1p-20f);
                     W = ni + (uint32_t)__float2int_rn(dr);      // 32 bits: a 64-bit conversion is an FP64 operation
-                    open = !(fabsf(__fsub_rn(rem, dr)) < __fsub_rn(0.5f, err)) || !(vvh < 2148000000.0f) || p > 900.0f;
+                    open = !(fabsf(__fsub_rn(rem, dr)) < __fsub_rn(0.5f, err)) || !(vvh < 2148000000.0f) ||
+                           __fsub_rn(F.lpre, p) < -1015.0f;      // (the Planck function a subnormal)
                 }
             }
             if (open)
@@ -991,7 +979,8 @@ cudaError_t launch_dust_emission(const DevCloud *dcl, int64_t n_leaf, const Temp
     const unsigned cap = std::max(1u, (unsigned)(grid_for((int64_t)1 << 40, 256) / fy));      // about 8 blocks per SM in all
     const int64_t tile = 256 * kDustLeaves;
     const dim3 g1((unsigned)std::min<int64_t>((n_leaf + tile - 1) / tile, cap), fy);
-    const dim3 g2((unsigned)std::min<int64_t>((n_leaf + 255) / 256, cap), fy);
+    // (the weight kernel holds five blocks an SM: one wave of them)
+    const dim3 g2((unsigned)std::min<int64_t>((n_leaf + 255) / 256, std::max(1u, cap * 5 / 8)), fy);
     dust_bound_kernel<<<g1, 256, 0, s>>>(dcl, n_leaf, tt, T, freq_lo, n_freq, lmax);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     dust_max_kernel<<<g1, 256, 0, s>>>(dcl, n_leaf, tt, T, freq_lo, n_freq, lmax, scratch_max);
