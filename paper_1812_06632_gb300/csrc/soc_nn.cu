@@ -105,6 +105,27 @@ __device__ __forceinline__ bool mbar_wait(uint32_t addr, uint32_t parity)
     return false;
 }
 
+// One MMA of kind::f16 (accumulator acc; operand descriptors as their low
+// words, the start addresses, and high words).  The issuing thread runs alone
+// at about one instruction in five cycles, so an MMA that takes the tensor
+// core 39 cycles leaves room for half a dozen: callers keep the low words in
+// registers and add to those only (the smem addresses stay below 2^18, so the
+// 14-bit field does not overflow).  kFirst: overwrite the accumulator if add
+// is 0; otherwise always add.
+template <bool kFirst = false>
+__device__ __forceinline__ void mma_f16(uint32_t acc, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
+                                        uint32_t idesc, uint32_t add = 1u)
+{
+    if (kFirst)
+        asm volatile("{\n .reg .pred p;\n .reg .b64 da, db;\n mov.b64 da, {%1, %2};\n mov.b64 db, {%3, %4};\n"
+                     " setp.ne.b32 p, %6, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n}\n"
+                     :: "r"(acc), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(add) : "memory");
+    else
+        asm volatile("{\n .reg .pred p;\n .reg .b64 da, db;\n mov.b64 da, {%1, %2};\n mov.b64 db, {%3, %4};\n"
+                     " setp.ne.b32 p, 1, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n}\n"
+                     :: "r"(acc), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc) : "memory");
+}
+
 // 16-byte asynchronous copy global -> shared through L1 (the weight gradient
 // reads its output gradient at three shifts); src_bytes = 0 writes zeros
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, uint32_t src_bytes)
@@ -140,6 +161,12 @@ struct ConvOut {
     const bf16 *mask;
     int m_stride, m_off, first_only;
 };
+
+ConvOut conv_out(const ConvArgs &a)
+{
+    return ConvOut{a.out, a.out_f32, a.bias, a.out_stride, a.out_off, a.relu, a.accumulate, a.mask, a.m_stride, a.m_off,
+                   a.first_only};
+}
 
 struct TmaConvArgs {
     int N, D, H, W, Cin, Cout;
@@ -693,7 +720,7 @@ struct WgradArgs {
     int gy_stride, gy_off;
     const bf16 *x;
     int x_stride, x_off;
-    float *part;                     // [gridDim.x][Cout][27][Cin]: each block's partial sums
+    float *part;                     // [chunks][Cout][27][Cin] weight sums, then [chunks n_ci][Cout] bias sums
     int N, D, H, W, Cin, Cout;
     // plan (wgrad_plan)
     int by, bxk, segs, tiles_y, n_boxes;
@@ -729,11 +756,18 @@ struct WgradArgs {
 // Warps 0-15 copy (16-byte cp.async; out-of-volume voxels are written as
 // zeros), one thread of warp 16 issues the MMAs, and warps 0-3 read the sums
 // out at the end.  The copies' address arithmetic is what bounds the kernel
-// (eight copying warps: 77 us at 64^3, 16 -> 16, against 20 us of MMAs).  A block takes the boxes [n_boxes b / chunks, n_boxes
+// at 64^3, 16 -> 16: 80 us, 72 without the MMAs, 46 without the
+// copies.  A block takes the boxes [n_boxes b / chunks, n_boxes
 // (b + 1) / chunks) and writes its sums to partial slice b;
 // reduce_partials_kernel adds the slices in order, so the result does not
 // depend on scheduling.  Rows of at most 8 voxels are taken in pairs (K = 16
 // is the descriptors' two 8-voxel cores, one row apart).
+//
+// The blocks also sum gy itself, the bias gradient (the n_ci blocks that share
+// a chunk and output channels take its boxes in turn): the copying warps add
+// up the unshifted rows in shared memory once a box has landed (a stage is
+// free again when the MMAs and these sums are done with it).  Kernels of
+// their own for it took 10 to 15 us a layer.
 // ---------------------------------------------------------------------------
 constexpr int kWgCopyWarps = 16;
 constexpr int kWgThreads = 32 * (kWgCopyWarps + 1);
@@ -768,7 +802,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv3d_wgrad_tc_kernel(const Wg
     if (tid == 0) {
         for (int k = 0; k < n_stages; ++k) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(smem_u32(&full[k])), "r"(kWgCopyWarps) : "memory");
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&empty[k])) : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(smem_u32(&empty[k])), "r"(kWgCopyWarps + 1) : "memory");
         }
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(done)) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -780,10 +814,16 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv3d_wgrad_tc_kernel(const Wg
     const uint32_t tmem = *tslot;
 
     const int n_ci = a.Cin / (8 * HN);
-    const int ci0 = ((int)blockIdx.y % n_ci) * 8 * HN, co0 = ((int)blockIdx.y / n_ci) * a.n_tile;
+    const int ci_tile = (int)blockIdx.y % n_ci;
+    const int ci0 = ci_tile * 8 * HN, co0 = ((int)blockIdx.y / n_ci) * a.n_tile;
     const int box0 = (int)((long long)a.n_boxes * blockIdx.x / gridDim.x);
     const int box1 = (int)((long long)a.n_boxes * (blockIdx.x + 1) / gridDim.x);
     const int nn = a.n_tile / 8;                           // channel groups of gy
+    // bias sums: copying thread -> channel group bias_g, voxels bias_v,
+    // bias_v + bias_lanes, ... of each box
+    const int bias_lanes = 32 * kWgCopyWarps / nn, bias_g = tid % nn, bias_v = tid / nn;
+    const bool bias_on = bias_v < bias_lanes;
+    float bias_sum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 
     if (warp < kWgCopyWarps) {
         // lane's first piece of a row of x and of gy (channel groups fastest),
@@ -793,34 +833,61 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv3d_wgrad_tc_kernel(const Wg
         const int a_src = ax * a.x_stride + ah * 8, a_step = (32 / HN) * a.x_stride;
         const int q0 = lane / nn, r0 = lane - q0 * nn, dq = 32 / nn, dr = 32 - dq * nn;
         int st = 0, issued = 0, told = 0;
+        int turn = (box0 + n_ci - ci_tile) % n_ci;         // 0: this block sums the next box's gy
         uint32_t ph = 0;
         // the oldest box not yet announced has landed: make it visible to the
-        // tensor cores and announce it
+        // tensor cores and announce it, add its bias sums
         auto announce = [&]() {
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
+            const int k = told % n_stages;
             if (lane == 0)
-                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_u32(&full[told % n_stages])) : "memory");
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_u32(&full[k])) : "memory");
+            if (turn == 0) {
+                if (!mbar_wait(smem_u32(&full[k]), (uint32_t)(told / n_stages) & 1u)) atomicExch(s_fail, 1);
+                const uint4 *const B = reinterpret_cast<const uint4 *>(smem + 256 + k * a.stage_bytes + a.a_bytes);
+                for (int y = 0, xq = bias_v; bias_on; xq += bias_lanes) {
+                    while (xq >= a.bxk) { xq -= a.bxk; ++y; }
+                    if (y >= a.by) break;
+                    const uint4 u = B[((3 * y + 1) * nn + bias_g) * a.bp + xq];
+                    const __nv_bfloat16 *h = reinterpret_cast<const __nv_bfloat16 *>(&u);
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) bias_sum[j] += __bfloat162float(h[j]);
+                }
+                __syncwarp();
+            }
+            if (lane == 0)
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_u32(&empty[k])) : "memory");
             ++told;
+            if (++turn == n_ci) turn = 0;
         };
+        // box coordinates, advanced by carries: decoding them by division
+        // and forming every row's address in 64 bits took longer than the
+        // copies themselves
+        int seg, ty, z;
+        long long nzy;                    // n D + z, the plane
+        {
+            int q = box0;
+            seg = q % a.segs; q /= a.segs;
+            ty = q % a.tiles_y; q /= a.tiles_y;
+            z = q % a.D;
+            nzy = q;
+        }
+        const long long x_row = (long long)a.W * a.x_stride, x_plane = a.H * x_row, gy_row = (long long)a.W * a.gy_stride;
         for (int box = box0; box < box1; ++box) {
             bool ok = !*fail;
             if (ok && issued >= n_stages) ok = mbar_wait(smem_u32(&empty[st]), ph ^ 1u);
             if (__any_sync(0xffffffffu, !ok)) { if (lane == 0) atomicExch(s_fail, 1); break; }
-            int q = box;
-            const int seg = q % a.segs; q /= a.segs;
-            const int ty = q % a.tiles_y; q /= a.tiles_y;
-            const int z = q % a.D, n = q / a.D;
             const int x0 = seg * a.bxk, y0 = ty * a.by;
             const uint32_t A0 = smem0 + (uint32_t)(st * a.stage_bytes), B0 = A0 + (uint32_t)a.a_bytes;
+            const long long row0 = nzy * a.H + y0;
+            const bf16 *const xb = a.x + row0 * x_row + (long long)x0 * a.x_stride + a.x_off + ci0;
+            const bf16 *const gb = a.gy + row0 * gy_row + a.gy_off + co0;
             const int wx = a.W - x0;                       // voxels of the rows left from x0 on
-            const int rows = 3 * (a.by + 2);
-            for (int r = warp; r < rows; r += kWgCopyWarps) {
+            for (int r = warp; r < 3 * (a.by + 2); r += kWgCopyWarps) {
                 const int yp = r / 3, zp = r - 3 * yp;
-                const int yy = y0 + yp - 1, zz = z + zp - 1;
-                const bool row = (unsigned)yy < (unsigned)a.H && (unsigned)zz < (unsigned)a.D;
-                const bf16 *const base = a.x + (row ? ((((long long)n * a.D + zz) * a.H + yy) * a.W + x0) * a.x_stride : 0LL) +
-                                         a.x_off + ci0;
+                const bool row = (unsigned)(y0 + yp - 1) < (unsigned)a.H && (unsigned)(z + zp - 1) < (unsigned)a.D;
+                const bf16 *const base = row ? xb + ((zp - 1) * x_plane + (yp - 1) * x_row) : a.x;
                 const int lim = row ? wx : 0;
                 uint32_t dst = A0 + (uint32_t)((yp * HN * 3 + zp) * a.wp) * 16u + a_dst;
                 int off = a_src;
@@ -833,11 +900,10 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv3d_wgrad_tc_kernel(const Wg
                 }
             }
             for (int r = warp; r < 3 * a.by; r += kWgCopyWarps) {
-                const int y = r / 3, c = r - 3 * y, yy = y0 + y;
-                const bool row = yy < a.H;
+                const int y = r / 3, c = r - 3 * y;
+                const bool row = y0 + y < a.H;
                 // shared voxel q is voxel x0 + q - (c - 1) of the row
-                const bf16 *const base = a.gy + (row ? (((long long)n * a.D + z) * a.H + yy) * a.W * a.gy_stride : 0LL) +
-                                         a.gy_off + co0;
+                const bf16 *const base = row ? gb + y * gy_row : a.gy;
                 const int sh = x0 - (c - 1), len = row ? a.W : 0;
                 const uint32_t dst = B0 + (uint32_t)(r * nn * a.bp) * 16u;
 #pragma unroll 4
@@ -847,6 +913,14 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv3d_wgrad_tc_kernel(const Wg
                                in ? 16u : 0u);
                     xq += dq; g += dr;
                     if (g >= nn) { g -= nn; ++xq; }
+                }
+            }
+            if (++seg == a.segs) {
+                seg = 0;
+                if (++ty == a.tiles_y) {
+                    ty = 0;
+                    ++nzy;
+                    if (++z == a.D) z = 0;
                 }
             }
             asm volatile("cp.async.commit_group;" ::: "memory");
@@ -865,6 +939,13 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv3d_wgrad_tc_kernel(const Wg
         const int a_row = HN * 3 * a.wp, b_row = 3 * nn * a.bp;          // in voxels of 16 bytes
         const uint32_t a_lbo = pair ? (uint32_t)a_row * 16u : 128u, b_lbo = pair ? (uint32_t)b_row * 16u : 128u;
         const int row_steps = pair ? 1 : a.bxk / 16, row_inc = pair ? 2 : 1;
+        const uint32_t a_inc = (uint32_t)(row_inc * a_row), b_inc = (uint32_t)(row_inc * b_row);
+        uint32_t acc_col[kTiles], t_off[kTiles];
+#pragma unroll
+        for (int t = 0; t < kTiles; ++t) {
+            acc_col[t] = tmem + (uint32_t)(t * 3 * a.n_tile);
+            t_off[t] = (uint32_t)(t * 16 * a.wp);
+        }
         int st = 0;
         uint32_t ph = 0, acc = 0;
         for (int box = box0; box < box1; ++box) {
@@ -876,18 +957,19 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv3d_wgrad_tc_kernel(const Wg
             const uint32_t A0 = smem0 + (uint32_t)(st * a.stage_bytes);
             const uint64_t da = smem_desc(A0, a_lbo, (uint32_t)a.wp * 16u);
             const uint64_t db = smem_desc(A0 + (uint32_t)a.a_bytes, b_lbo, (uint32_t)a.bp * 16u);
+            const uint32_t a_hi = (uint32_t)(da >> 32), b_hi = (uint32_t)(db >> 32);
+            uint32_t a_row_lo = (uint32_t)da, b_row_lo = (uint32_t)db;
             for (int y = 0; y < rows; y += row_inc) {
-                for (int s = 0; s < row_steps; ++s) {
-                    const uint64_t ad = da + (uint32_t)(y * a_row + s * 16), bd = db + (uint32_t)(y * b_row + s * 16);
 #pragma unroll
-                    for (int t = 0; t < kTiles; ++t) {
-                        asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                                     " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-                                     :: "r"(tmem + (uint32_t)(t * 3 * a.n_tile)), "l"(ad + (uint32_t)(t * 16 * a.wp)),
-                                        "l"(bd), "r"(idesc), "r"(acc) : "memory");
-                    }
+                for (int s = 0; s < 4; ++s) {
+                    if (s >= row_steps) break;
+#pragma unroll
+                    for (int t = 0; t < kTiles; ++t)
+                        mma_f16<true>(acc_col[t], a_row_lo + t_off[t] + 16u * s, a_hi, b_row_lo + 16u * s, b_hi, idesc, acc);
                     acc = 1;
                 }
+                a_row_lo += a_inc;
+                b_row_lo += b_inc;
             }
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
                          :: "r"(smem_u32(&empty[st])) : "memory");
@@ -904,9 +986,31 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv3d_wgrad_tc_kernel(const Wg
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (!ok_run) {
         if (tid == 0) atomicExch(&g_tc_error, 1);
-    } else if (warp < 4) {
+    }
+    const long long n_w = (long long)a.Cout * 27 * a.Cin;
+    float *const slice = a.part + blockIdx.x * n_w;
+    if (ok_run) {
+        // the stages are free: sums over the copying threads, first in
+        // 512 / n_tile rows, then over the rows in order
+        float *const s_sum = reinterpret_cast<float *>(smem + 256);
+        if (tid < 32 * kWgCopyWarps)
+            for (int j = 0; j < 8; ++j) s_sum[tid * 9 + j] = bias_on ? bias_sum[j] : 0.f;
+        __syncthreads();
+        const int rows = 32 * kWgCopyWarps / a.n_tile, c = tid % a.n_tile, row = tid / a.n_tile;
+        float t = 0.f;
+        if (row < rows)
+            for (int k = row; k < bias_lanes; k += rows) t += s_sum[(k * nn + c / 8) * 9 + c % 8];
+        __syncthreads();
+        if (row < rows) s_sum[tid] = t;
+        __syncthreads();
+        if (tid < a.n_tile) {
+            t = 0.f;
+            for (int k = 0; k < rows; ++k) t += s_sum[k * a.n_tile + tid];
+            a.part[gridDim.x * n_w + ((long long)blockIdx.x * n_ci + ci_tile) * a.Cout + co0 + tid] = t;
+        }
+    }
+    if (ok_run && warp < 4) {
         // accumulator row 8 (g mod 16) + c of tile g / 16: group g = (dy HN + h) 3 + dz, channel ci0 + 8 h + c
-        float *const slice = a.part + (long long)blockIdx.x * a.Cout * 27 * a.Cin;
 #pragma unroll
         for (int t = 0; t < kTiles; ++t) {
             const int g = 16 * t + tid / 8, dz = g % 3, h = (g / 3) % HN, dy = g / (3 * HN);
@@ -931,84 +1035,55 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv3d_wgrad_tc_kernel(const Wg
     }
 }
 
-// out[i] += sum_{k < n_parts} part[k * n + i]: a block takes 256 / S elements;
+// gw[i] += sum_{k < n_parts} part[k n_w + i], and (gb not null) gb[c] += sum_{k
+// < n_ci n_parts} of the bias sums behind them: a block takes 256 / S elements;
 // thread row s of its S adds the parts s, s + S, ... in order, then the rows
 // are added in order (the same order on every run).  With one row everywhere
 // the parts of the small layers formed chains of up to 152 dependent loads.
 template <int S>
-__global__ void __launch_bounds__(256) reduce_partials_kernel(const float *part, int n_parts, long long n, float *out)
+__global__ void __launch_bounds__(256) reduce_partials_kernel(const float *part, int n_parts, int n_ci, long long n_w,
+                                                              int n_b, float *gw, float *gb)
 {
     constexpr int E = 256 / S;
     __shared__ float s_sum[S][E + 1];
     const int e = threadIdx.x % E, s = threadIdx.x / E;
     const long long i = (long long)blockIdx.x * E + e;
+    const bool weight = i < n_w;
+    float *const out = weight ? gw + i : (i < n_w + n_b && gb ? gb + (i - n_w) : nullptr);
+    const float *const src = weight ? part + i : part + n_parts * n_w + (i - n_w);
+    const long long stride = weight ? n_w : n_b;
+    const int parts = weight ? n_parts : n_parts * n_ci;
     float v = 0.f;
-    if (i < n) {
+    if (out) {
 #pragma unroll 8
-        for (int k = s; k < n_parts; k += S) v += part[(long long)k * n + i];
+        for (int k = s; k < parts; k += S) v += src[k * stride];
     }
     if (S == 1) {
-        if (i < n) out[i] += v;
+        if (out) *out += v;
         return;
     }
     s_sum[s][e] = v;
     __syncthreads();
-    if (s == 0 && i < n) {
+    if (s == 0 && out) {
         float t = 0.f;
 #pragma unroll
         for (int k = 0; k < S; ++k) t += s_sum[k][e];
-        out[i] += t;
+        *out += t;
     }
 }
 
 // Rows by size: enough threads to fill the chip (about 300 000), no more rows
 // than parts.
-inline void reduce_partials(const float *part, int n_parts, long long n, float *out, cudaStream_t s)
+inline void reduce_partials(const float *part, int n_parts, int n_ci, long long n_w, int n_b, float *gw, float *gb,
+                            cudaStream_t s)
 {
-    if (n >= 300000 || n_parts < 8) reduce_partials_kernel<1><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(part, n_parts, n, out);
-    else if (n >= 10000 || n_parts < 32) reduce_partials_kernel<8><<<(unsigned)((n + 31) / 32), 256, 0, s>>>(part, n_parts, n, out);
-    else reduce_partials_kernel<64><<<(unsigned)((n + 3) / 4), 256, 0, s>>>(part, n_parts, n, out);
-}
-
-// Bias gradient, per block: part[blockIdx.x][c] = sum over the block's voxels
-// of gy[v][c] (BF16 gradient, dense C channels).  A thread takes the 8
-// channels of group threadIdx.x % (C / 8) (one 16-byte load a voxel), the
-// threads of a group every 256 / (C / 8)-th voxel; reduce_partials_kernel
-// adds the blocks' sums.
-__global__ void __launch_bounds__(256) bias_grad_kernel(const bf16 *gy, int C, long long V, long long vox_per_block,
-                                                        float *part)
-{
-    __shared__ float s_part[256][9];
-    const int ng = C / 8, nv = 256 / ng, g = threadIdx.x % ng, lane_v = threadIdx.x / ng;
-    const long long vb = (long long)blockIdx.x * vox_per_block;
-    const long long ve = vb + vox_per_block < V ? vb + vox_per_block : V;
-    float sum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    if (lane_v < nv) {
-#pragma unroll 4
-        for (long long v = vb + lane_v; v < ve; v += nv) {
-            const uint4 u = *reinterpret_cast<const uint4 *>(gy + v * C + 8 * g);
-            const __nv_bfloat16 *h = reinterpret_cast<const __nv_bfloat16 *>(&u);
-#pragma unroll
-            for (int j = 0; j < 8; ++j) sum[j] += __bfloat162float(h[j]);
-        }
-    }
-#pragma unroll
-    for (int j = 0; j < 8; ++j) s_part[threadIdx.x][j] = sum[j];
-    __syncthreads();
-    // channel c from its nv voxel lanes: 256 / C threads each take every
-    // (256 / C)-th of them, then their sums are added in order
-    const int c = threadIdx.x % C, q = threadIdx.x / C, nq = 256 / C;
-    float t = 0.f;
-    if (q < nq)
-        for (int k = q; k < nv; k += nq) t += s_part[k * ng + c / 8][c % 8];
-    __syncthreads();
-    if (q < nq) s_part[threadIdx.x][8] = t;
-    __syncthreads();
-    if (q == 0) {
-        t = 0.f;
-        for (int k = 0; k < nq; ++k) t += s_part[k * C + c][8];
-        part[(long long)blockIdx.x * C + c] = t;
-    }
+    const long long n = n_w + n_b;
+    auto run = [&](auto kernel, int per_block) {
+        kernel<<<(unsigned)((n + per_block - 1) / per_block), 256, 0, s>>>(part, n_parts, n_ci, n_w, n_b, gw, gb);
+    };
+    if (n >= 300000 || n_parts < 8) run(reduce_partials_kernel<1>, 256);
+    else if (n >= 10000 || n_parts < 32) run(reduce_partials_kernel<8>, 32);
+    else run(reduce_partials_kernel<64>, 4);
 }
 
 // Kernels over the voxels of a volume N x D x H x W: blockIdx.y (strided by
@@ -1295,6 +1370,56 @@ inline dim3 grid_rows(int row_threads, long long rows)
 }
 
 
+// Limits of the current device, asked for once per device: the attribute
+// queries and kernel attributes of every launch made small convolutions wait
+// for the host.
+constexpr int kMaxDevices = 64;
+struct DeviceLimits { int sms = 148, sm_smem = 233472, blk_max = 232448; };
+
+inline int current_device()
+{
+    int dev = 0;
+    cudaGetDevice(&dev);
+    return dev < 0 || dev >= kMaxDevices ? 0 : dev;
+}
+
+inline const DeviceLimits &device_limits()
+{
+    static DeviceLimits lim[kMaxDevices];
+    static std::once_flag once[kMaxDevices];
+    const int dev = current_device();
+    std::call_once(once[dev], [dev] {
+        cudaDeviceGetAttribute(&lim[dev].sms, cudaDevAttrMultiProcessorCount, dev);
+        cudaDeviceGetAttribute(&lim[dev].sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+        cudaDeviceGetAttribute(&lim[dev].blk_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    });
+    return lim[dev];
+}
+
+// Lets a kernel have all the shared memory a block may have (carveout: and
+// prefers shared memory to L1, so that the planned blocks fit an SM), once
+// per device; regs: its registers per thread.
+template <auto Kernel, bool kCarveout>
+cudaError_t kernel_setup(int *regs = nullptr)
+{
+    static cudaError_t err[kMaxDevices];
+    static int n_regs[kMaxDevices];
+    static std::once_flag once[kMaxDevices];
+    const int dev = current_device();
+    std::call_once(once[dev], [dev] {
+        cudaFuncAttributes fa;
+        cudaError_t e = cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, device_limits().blk_max);
+        if (e == cudaSuccess && kCarveout)
+            e = cudaFuncSetAttribute(Kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                     (int)cudaSharedmemCarveoutMaxShared);
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, Kernel);
+        if (e == cudaSuccess) n_regs[dev] = fa.numRegs;
+        err[dev] = e;
+    });
+    if (regs) *regs = n_regs[dev];
+    return err[dev];
+}
+
 // Output channels per block of the tensor-core convolution: a multiple of
 // 16 dividing C_out, at most 256, narrowed (down to 16) while the blocks
 // would cover fewer than half the SMs (narrow tiles re-read A, so they only
@@ -1338,11 +1463,7 @@ cudaError_t tma_launch(const ConvArgs &a, cudaStream_t s)
     if (!encode) return cudaErrorNotSupported;
     const uintptr_t in_addr = reinterpret_cast<uintptr_t>(a.in + a.in_off);
     if ((in_addr & 15u) || (a.in_stride % 8) || (reinterpret_cast<uintptr_t>(a.w) & 15u)) return cudaErrorInvalidValue;
-    int dev = 0, sms = 148, sm_smem = 0, blk_max = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-    cudaDeviceGetAttribute(&blk_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    const int sms = device_limits().sms, sm_smem = device_limits().sm_smem, blk_max = device_limits().blk_max;
     TmaConvArgs t{};
     t.N = a.N; t.D = a.D; t.H = a.H; t.W = a.W; t.Cin = a.Cin; t.Cout = a.Cout;
     t.bx = std::min(a.W, 128);
@@ -1353,8 +1474,7 @@ cudaError_t tma_launch(const ConvArgs &a, cudaStream_t s)
     t.tiles_y = (a.H + t.by - 1) / t.by;
     t.tiles_z = (a.D + t.bz - 1) / t.bz;
     const long long tiles = (long long)t.tiles_x * t.tiles_y * t.tiles_z * ((a.N + t.bn - 1) / t.bn);
-    t.o = ConvOut{a.out, a.out_f32, a.bias, a.out_stride, a.out_off, a.relu, a.accumulate, a.mask, a.m_stride,
-                  a.m_off, a.first_only};
+    t.o = conv_out(a);
     const int n_tile = tc_n_tile(a.Cout, tiles, sms);
     constexpr CUtensorMapSwizzle sw = KC == 16 ? CU_TENSOR_MAP_SWIZZLE_32B
                                     : (KC == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B);
@@ -1386,32 +1506,30 @@ cudaError_t tma_launch(const ConvArgs &a, cudaStream_t s)
     uint32_t cols = 32;
     while ((int)cols < 2 * n_tile) cols <<= 1;
     if (cols > 512) return cudaErrorInvalidValue;
-    // blocks per SM: at most what 512 columns of tensor memory hold, and 8;
-    // the rest of the SM's shared memory split among them as stages, 2 to 8
-    const int per_sm = std::min(8, std::min(512 / (int)cols, 2048 / kConvThreads));
+    // blocks per SM: what the grid has for each, at most what 512 columns of
+    // tensor memory hold, and 8; the SM's shared memory split among them as
+    // stages, 2 to 24 (a step is a fraction of a TMA round trip, so few blocks
+    // want many: the 8^3 layers, 128 blocks, ran 2 stages each)
+    const long long blocks = tiles * (a.Cout / n_tile);
+    const int per_sm = (int)std::min<long long>(std::min(8, std::min(512 / (int)cols, 2048 / kConvThreads)),
+                                                (blocks + sms - 1) / sms);
     const int stage_bytes = (128 + n_tile) * KC * 2;
-    const int fixed = 1024 + 8 * (2 * 8 + 5) + 8;     // alignment, barriers, slot and flag
-    int stages = (sm_smem / per_sm - 1024 - fixed) / stage_bytes;
-    stages = stages < 2 ? 2 : (stages > 8 ? 8 : stages);
+    const int fixed = 1024 + 8 * (2 * 24 + 5) + 8;    // alignment, barriers, slot and flag
+    int stages = (std::min(sm_smem / per_sm - 1024, blk_max) - fixed) / stage_bytes;
+    stages = stages < 2 ? 2 : (stages > 24 ? 24 : stages);
     const int need = 1024 + stages * stage_bytes + 8 * (2 * stages + 5) + 8;
     if (need > blk_max) return cudaErrorInvalidValue;
     // padded so that no more than per_sm blocks are resident on an SM
     const int pad = sm_smem / (per_sm + 1) + 1024;
     int bytes = need > pad ? need : pad;
     if (bytes > blk_max) bytes = blk_max;
-    cudaError_t e = cudaFuncSetAttribute(conv3d_tma_kernel<KC>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e != cudaSuccess) return e;
-    // all of the SM's unified memory as shared memory, so that per_sm blocks fit
-    e = cudaFuncSetAttribute(conv3d_tma_kernel<KC>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             (int)cudaSharedmemCarveoutMaxShared);
-    if (e != cudaSuccess) return e;
     // blocks an SM holds, from the kernel's registers (the runtime's occupancy
     // query answers 1 for any kernel that allocates tensor memory); more
     // blocks than the SMs hold only run later, each still walking its boxes
-    cudaFuncAttributes fa;
-    e = cudaFuncGetAttributes(&fa, conv3d_tma_kernel<KC>);
+    int regs = 0;
+    const cudaError_t e = kernel_setup<conv3d_tma_kernel<KC>, true>(&regs);
     if (e != cudaSuccess) return e;
-    const int warp_regs = ((fa.numRegs + 7) / 8) * 8 * 32;
+    const int warp_regs = ((regs + 7) / 8) * 8 * 32;
     const int reg_blocks = 65536 / (warp_regs * (kConvThreads / 32));
     const int occ = std::max(1, std::min(per_sm, reg_blocks));
     const int grid_y = a.Cout / n_tile;
@@ -1493,8 +1611,7 @@ cudaError_t slab_launch(const ConvArgs &a, const SlabPlan &p, int sms, cudaStrea
     t.by = p.by; t.bz = p.bz; t.g = 128 / a.W; t.gyn = p.gyn; t.n_acc = p.n_acc;
     t.tiles_y = (a.H + p.by - 1) / p.by;
     t.tiles_z = (a.D + p.bz - 1) / p.bz;
-    t.o = ConvOut{a.out, a.out_f32, a.bias, a.out_stride, a.out_off, a.relu, a.accumulate, a.mask, a.m_stride,
-                  a.m_off, a.first_only};
+    t.o = conv_out(a);
     constexpr CUtensorMapSwizzle sw = KC == 16 ? CU_TENSOR_MAP_SWIZZLE_32B
                                     : (KC == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B);
     CUtensorMap map_in, map_w;
@@ -1522,15 +1639,10 @@ cudaError_t slab_launch(const ConvArgs &a, const SlabPlan &p, int sms, cudaStrea
     }
     uint32_t cols = 32;
     while ((int)cols < 2 * p.n_acc * p.n_tile) cols <<= 1;
-    cudaError_t e = cudaFuncSetAttribute(conv3d_slab_kernel<KC, NACC>, cudaFuncAttributeMaxDynamicSharedMemorySize, p.bytes);
+    int regs = 0;
+    const cudaError_t e = kernel_setup<conv3d_slab_kernel<KC, NACC>, true>(&regs);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(conv3d_slab_kernel<KC, NACC>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             (int)cudaSharedmemCarveoutMaxShared);
-    if (e != cudaSuccess) return e;
-    cudaFuncAttributes fa;
-    e = cudaFuncGetAttributes(&fa, conv3d_slab_kernel<KC, NACC>);
-    if (e != cudaSuccess) return e;
-    const int warp_regs = ((fa.numRegs + 7) / 8) * 8 * 32;
+    const int warp_regs = ((regs + 7) / 8) * 8 * 32;
     const int occ = std::max(1, std::min(p.per_sm, 65536 / (warp_regs * (kConvThreads / 32))));
     const int grid_y = a.Cout / p.n_tile;
     const long long n_boxes = (long long)t.tiles_y * t.tiles_z * a.N;
@@ -1545,11 +1657,7 @@ cudaError_t slab_launch(const ConvArgs &a, const SlabPlan &p, int sms, cudaStrea
 // chunks of 64, 32 or 16 input channels (the largest dividing C_in).
 cudaError_t conv_launch(const ConvArgs &a, cudaStream_t s)
 {
-    int dev = 0, sms = 148, sm_smem = 0, blk_max = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-    cudaDeviceGetAttribute(&blk_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    const int sms = device_limits().sms, sm_smem = device_limits().sm_smem, blk_max = device_limits().blk_max;
     SlabPlan p{};
     if (slab_plan(a, sms, sm_smem, blk_max, p)) {
         if (p.kc == 32)
@@ -1598,7 +1706,7 @@ inline bool wgrad_plan(int N, int D, int H, int W, int Cin, int Cout, int sms, i
         p.stage_bytes = (p.a_bytes + by * 3 * (nt / 8) * p.bp * 16 + 127) / 128 * 128;
         const int pad = (wgrad_tiles(hn) * 16 - 9 * hn) * p.wp * 16;     // what the last tile reads past its groups
         p.stages = std::min(6, (blk_max - 256 - pad) / p.stage_bytes);
-        p.bytes = 256 + p.stages * p.stage_bytes + pad;
+        p.bytes = std::max(256 + p.stages * p.stage_bytes + pad, 256 + 32 * kWgCopyWarps * 9 * 4);
         p.by = by;
         return p.stages >= 3;                // copies of one box, one landing, MMAs of one
     };
@@ -1656,78 +1764,43 @@ inline bool wgrad_plan(int N, int D, int H, int W, int Cin, int Cout, int sms, i
     return true;
 }
 
-inline int device_sms()
+// The plan on the current device (false: none).
+inline bool wgrad_plan_here(int N, int D, int H, int W, int Cin, int Cout, WgradPlan &p)
 {
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return sms;
+    return wgrad_plan(N, D, H, W, Cin, Cout, device_limits().sms, device_limits().blk_max, p);
 }
 
-inline int device_block_smem()
+// Floats of partial sums a weight gradient needs.
+inline long long wgrad_part_floats(const WgradPlan &p, int Cin, int Cout)
 {
-    int dev = 0, v = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    return v;
-}
-
-// Floats of partial sums a weight gradient of this shape needs.
-inline long long wgrad_part_floats(int N, int D, int H, int W, int Cin, int Cout)
-{
-    WgradPlan p;
-    if (!wgrad_plan(N, D, H, W, Cin, Cout, device_sms(), device_block_smem(), p)) return 0;
-    return (long long)p.chunks * Cout * 27 * Cin;
+    return (long long)p.chunks * (Cout * 27LL * Cin + (long long)(Cin / (8 * p.hn)) * Cout);
 }
 
 template <int HN>
 cudaError_t wgrad_start(const WgradArgs &a, const WgradPlan &p, cudaStream_t s)
 {
-    cudaError_t e = cudaFuncSetAttribute(conv3d_wgrad_tc_kernel<HN>, cudaFuncAttributeMaxDynamicSharedMemorySize, p.bytes);
+    const cudaError_t e = kernel_setup<conv3d_wgrad_tc_kernel<HN>, false>();
     if (e != cudaSuccess) return e;
     conv3d_wgrad_tc_kernel<HN><<<dim3((unsigned)p.chunks, (unsigned)p.combos), kWgThreads, p.bytes, s>>>(a);
     return cudaGetLastError();
 }
 
-// gw[Cout][27][Cin] += sum_v gy[v] x[v + tap]: partial sums per chunk of
-// boxes into part (part_floats available), then their ordered sum into gw.
-cudaError_t wgrad_launch(const WgradArgs &a0, float *gw, long long part_floats, cudaStream_t s)
+// gw[Cout][27][Cin] += sum_v gy[v] x[v + tap] and (gb not null) gb[Cout] +=
+// sum_v gy[v]: partial sums per chunk of boxes into part (part_floats
+// available), then their ordered sums.
+cudaError_t wgrad_launch(const WgradArgs &a0, const WgradPlan &p, float *gw, float *gb, long long part_floats,
+                         cudaStream_t s)
 {
     WgradArgs a = a0;
-    WgradPlan p;
-    if (!wgrad_plan(a.N, a.D, a.H, a.W, a.Cin, a.Cout, device_sms(), device_block_smem(), p)) return cudaErrorInvalidValue;
     const long long n_w = (long long)a.Cout * 27 * a.Cin;
-    if (p.chunks * n_w > part_floats) return cudaErrorInvalidValue;
+    if (wgrad_part_floats(p, a.Cin, a.Cout) > part_floats) return cudaErrorInvalidValue;
     a.by = p.by; a.bxk = p.bxk; a.segs = p.segs; a.tiles_y = (a.H + p.by - 1) / p.by; a.n_boxes = p.n_boxes;
     a.wp = p.wp; a.bp = p.bp; a.n_tile = p.n_tile; a.a_bytes = p.a_bytes; a.stage_bytes = p.stage_bytes;
     a.n_stages = p.stages; a.tmem_cols = p.cols;
     const cudaError_t e = p.hn == 8 ? wgrad_start<8>(a, p, s) : p.hn == 4 ? wgrad_start<4>(a, p, s)
                         : p.hn == 2 ? wgrad_start<2>(a, p, s) : wgrad_start<1>(a, p, s);
     if (e != cudaSuccess) return e;
-    reduce_partials(a.part, p.chunks, n_w, gw, s);
-    return cudaGetLastError();
-}
-
-// Voxels per block of the bias gradient: at least 16 per voxel lane, and at
-// most about 600 blocks (4 per SM), so that few partial sums are left.
-inline long long bias_vox(long long V, int C)
-{
-    const long long lanes = 256 / (C / 8);
-    return std::max(16 * lanes, (V + 607) / 608);
-}
-
-inline long long bias_part_floats(long long V, int C) { return (V + bias_vox(V, C) - 1) / bias_vox(V, C) * C; }
-
-// gb[C] += sum_v gy[v]: per-block sums into part, then their sum in a fixed
-// order.
-cudaError_t bias_grad_launch(const bf16 *gy, int C, long long V, float *gb, float *part, long long part_floats,
-                             cudaStream_t s)
-{
-    if (C < 8 || C % 8 || C > 256) return cudaErrorInvalidValue;
-    const long long vox = bias_vox(V, C), blocks = (V + vox - 1) / vox;
-    if (blocks * C > part_floats || blocks > 0x7FFFFFFF) return cudaErrorInvalidValue;
-    bias_grad_kernel<<<(unsigned)blocks, 256, 0, s>>>(gy, C, V, vox, part);
-    reduce_partials(part, (int)blocks, C, gb, s);
+    reduce_partials(a.part, p.chunks, a.Cin / (8 * p.hn), n_w, a.Cout, gw, gb, s);
     return cudaGetLastError();
 }
 
@@ -1801,6 +1874,7 @@ struct Net {
     Buf<bf16> g16[2];
     Buf<double> loss, loss_part;
     Buf<float> part;              // per-block partial sums of the weight and bias gradients
+    WgradPlan wplan[kLayers];
 
     float *bias(int l) { return par.p + bias_off(l); }
     bf16 *w16(int l) { return par16.p + weight_off(l); }
@@ -1908,13 +1982,11 @@ struct GradOut {
 soc_status bwd(Net &n, int l, const bf16 *gy, const bf16 *x, int S, const GradOut &g, cudaStream_t s)
 {
     const int Cin = kSpec[l].cin, Cout = kSpec[l].cout;
-    const long long V = (long long)n.batch * S * S * S;
     WgradArgs wa;
     memset(&wa, 0, sizeof wa);
     wa.gy = gy; wa.gy_stride = Cout; wa.x = x; wa.x_stride = Cin;
     wa.part = n.part.p; wa.N = n.batch; wa.D = S; wa.H = S; wa.W = S; wa.Cin = Cin; wa.Cout = Cout;
-    NNCK(wgrad_launch(wa, n.grad.p + weight_off(l), (long long)n.part.n, s));
-    NNCK(bias_grad_launch(gy, Cout, V, n.grad.p + bias_off(l), n.part.p, (long long)n.part.n, s));
+    NNCK(wgrad_launch(wa, n.wplan[l], n.grad.p + weight_off(l), n.grad.p + bias_off(l), (long long)n.part.n, s));
     if (g.f32 || g.b16) {
         ConvArgs a = conv_args(gy, Cout, 0, n.wt.p + weight_off(l), nullptr, n.batch, S, Cout, Cin, 0);
         a.out_f32 = g.f32; a.out = g.b16; a.out_stride = Cin;
@@ -2039,9 +2111,9 @@ soc_status soc_unet_create(int device, int batch, int side, int n_inputs, int *n
         long long need = 0;
         for (int l = 0; l < kLayers; ++l) {
             const int lev = l < 2 ? 0 : l < 4 ? 1 : l < 6 ? 2 : l < 8 ? 3 : l < 10 ? 2 : l < 12 ? 1 : 0;
-            const long long V = n->V0 >> (3 * lev);
-            need = std::max(need, wgrad_part_floats(batch, side >> lev, side >> lev, side >> lev, kSpec[l].cin, kSpec[l].cout));
-            need = std::max(need, bias_part_floats(V, kSpec[l].cout));
+            if (!wgrad_plan_here(batch, side >> lev, side >> lev, side >> lev, kSpec[l].cin, kSpec[l].cout, n->wplan[l]))
+                e = cudaErrorInvalidValue;
+            need = std::max(need, wgrad_part_floats(n->wplan[l], kSpec[l].cin, kSpec[l].cout));
         }
         A(n->part, (size_t)need);
     }
@@ -2181,8 +2253,10 @@ soc_status soc_nn_conv3d_wgrad(const void *gy, const void *x, int N, int D, int 
 {
     if (!gy || !x || !gw || Cin % 16 || Cout % 16 || N < 1 || D < 1 || H < 1 || W < 1) return SOC_ERR_ARG;
     cudaStream_t s = (cudaStream_t)stream;
-    const long long V = (long long)N * D * H * W;
-    const long long need = std::max(wgrad_part_floats(N, D, H, W, Cin, Cout), bias_part_floats(V, Cout));
+    WgradPlan plan;
+    if (!wgrad_plan_here(N, D, H, W, Cin, Cout, plan)) return SOC_ERR_CUDA;
+    if (gb && Cout > 256) return SOC_ERR_CUDA;
+    const long long need = wgrad_part_floats(plan, Cin, Cout);
     // partial sums in a library-owned workspace of this device (grown on
     // demand; calls on one device share it and are ordered by the caller)
     static std::mutex ws_mutex;
@@ -2205,8 +2279,7 @@ soc_status soc_nn_conv3d_wgrad(const void *gy, const void *x, int N, int D, int 
     memset(&wa, 0, sizeof wa);
     wa.gy = (const bf16 *)gy; wa.gy_stride = Cout; wa.x = (const bf16 *)x; wa.x_stride = Cin; wa.part = w.p;
     wa.N = N; wa.D = D; wa.H = H; wa.W = W; wa.Cin = Cin; wa.Cout = Cout;
-    NNCK(wgrad_launch(wa, gw, (long long)w.n, s));
-    if (gb) NNCK(bias_grad_launch((const bf16 *)gy, Cout, V, gb, w.p, (long long)w.n, s));
+    NNCK(wgrad_launch(wa, plan, gw, gb, (long long)w.n, s));
     return SOC_OK;
 }
 
