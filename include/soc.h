@@ -658,14 +658,15 @@ soc_status soc_nn_seed_features(const float *d_T, const float *d_T_prev, const f
 soc_status soc_set_launch(soc_ctx *ctx, int threads_per_block, int blocks_per_sm, int chunk);
 /* A warp refills its idle lanes with new packages once at least
  * min_idle_lanes (1..32) of its 32 lanes are idle (or all are): emission then
- * runs for several lanes together instead of one lane at a time.  Results do
- * not depend on it. */
+ * runs for several lanes together instead of one lane at a time.  Not set: 8,
+ * and 14 for launches of dust packages alone.  Results do not depend on it. */
 soc_status soc_set_refill(soc_ctx *ctx, int min_idle_lanes);
 /* A lane whose package has to scatter waits until min_lanes (1..32) lanes of
  * its warp wait too (or every active lane does); the warp then draws their
  * new directions together instead of diverging on every scattering.  Each
  * package's draws and operations keep their order: results do not depend
- * on it. */
+ * on it.  Not set: 8, and 4 for launches of dust packages alone or of several
+ * clouds. */
 soc_status soc_set_scatter_batch(soc_ctx *ctx, int min_lanes);
 /* Step cap per package (default 10^7); packages beyond it are ended with
  * their weight deposited and counted in stats[1]. */

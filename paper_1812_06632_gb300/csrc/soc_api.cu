@@ -83,6 +83,7 @@ struct BatchHost {
     uint64_t total = 0;
     HotCloud hot{};
     int32_t regular = 0;
+    bool dust = false;
     DevBuf<DevItem> items;
     DevBuf<uint64_t> prefix;
     DevBuf<unsigned long long> counter;
@@ -125,7 +126,8 @@ struct soc_ctx {
     DevBuf<int64_t> b_tally, b_self, b_stats;
     DevBuf<double> b_maxdT;
     // launch
-    int tpb = 256, bps = 4, chunk = 16, refill_min = 8, scatter_min = 8;   // autotuned on the 128^3 x 64 nu workload
+    int tpb = 256, bps = 4, chunk = 16;    // autotuned on the 128^3 x 64 nu workload
+    int refill_min = 0, scatter_min = 0;   // 0: by the kind of launch (launch_thresholds)
     uint32_t max_steps = 10000000u;
     int sms = 0;
     int occ[2][2][8] = {};        // resident blocks/SM per (regular grid, build, threads/32), from soc_create
@@ -873,6 +875,28 @@ static int32_t all_regular(const soc_ctx *ctx, const soc_batch_item *items, int 
     return 1;
 }
 
+// True when every item emits dust packages.
+static bool all_dust(const soc_batch_item *items, int n_items)
+{
+    for (int i = 0; i < n_items; ++i)
+        if (items[i].source != SOC_SRC_DUST) return false;
+    return true;
+}
+
+// How many idle lanes a warp refills at once and how many waiting ones it
+// scatters at once, unless the caller has set them.  Dust packages live a few
+// steps, so a warp emits all the time and pays for emitting for few lanes:
+// three 64^3 clouds' dust iterations took 51.5 ms with 8 and 8, 47.6 with 12
+// and 4, 47.1 with 16 and 4; a weighted octree iteration 33.6, 32.8 and 33.0.
+// Background and point packages: 60.1 ms with 8 and 8 on one 128^3 cloud (60.4
+// with 10, 61.3 with 8 and 4), 42.9 and 42.0 with 8 and 4 on twelve clouds, of
+// which thick ones scatter often.
+static void launch_thresholds(const soc_ctx *ctx, TraceParams &P, bool dust)
+{
+    P.refill_min = ctx->refill_min > 0 ? ctx->refill_min : (dust ? 14 : 8);
+    P.scatter_min = ctx->scatter_min > 0 ? ctx->scatter_min : (dust || !P.hot.cell ? 4 : 8);
+}
+
 // Launch shape of the tracer for P.total work indices, and the share of the
 // remaining work a warp takes at a time (2^-take_shift, the power of two at
 // or below half a warp's even share).
@@ -958,9 +982,8 @@ soc_status soc_simulate_frequency_batch_ex(soc_ctx *ctx, const soc_batch_item *i
         P.n_items = n_items;
         P.max_steps = ctx->max_steps;
         P.chunk = ctx->chunk;
-        P.refill_min = ctx->refill_min;
-        P.scatter_min = ctx->scatter_min;
         P.hot = one_cloud(ctx, items, n_items);
+        launch_thresholds(ctx, P, all_dust(items, n_items));
         P.regular = all_regular(ctx, items, n_items);
         int grid = 1, variant = 3;
         launch_geometry(ctx, P, grid, variant);
@@ -986,6 +1009,7 @@ soc_status soc_batch_create(soc_ctx *ctx, const soc_batch_item *items, int n_ite
         b->total = prefix[n_items];
         b->hot = one_cloud(ctx, items, n_items);
         b->regular = all_regular(ctx, items, n_items);
+        b->dust = all_dust(items, n_items);
         cudaError_t e = cudaSuccess;
         if ((e = b->items.alloc(n_items)) != cudaSuccess || (e = b->prefix.alloc(n_items + 1)) != cudaSuccess ||
             (e = b->counter.alloc(1)) != cudaSuccess ||
@@ -1032,9 +1056,8 @@ soc_status soc_batch_launch(soc_ctx *ctx, int batch_id, int64_t *d_tally, int64_
         P.n_items = b.n_items;
         P.max_steps = ctx->max_steps;
         P.chunk = ctx->chunk;
-        P.refill_min = ctx->refill_min;
-        P.scatter_min = ctx->scatter_min;
         P.hot = b.hot;
+        launch_thresholds(ctx, P, b.dust);
         P.regular = b.regular;
         int grid = 1, variant = 3;
         launch_geometry(ctx, P, grid, variant);
@@ -1966,9 +1989,8 @@ extern "C" soc_status soc_simulate_frequency_batch_noalloc(soc_ctx *ctx, const s
         P.n_items = n_items;
         P.max_steps = ctx->max_steps;
         P.chunk = ctx->chunk;
-        P.refill_min = ctx->refill_min;
-        P.scatter_min = ctx->scatter_min;
         P.hot = one_cloud(ctx, items, n_items);
+        launch_thresholds(ctx, P, all_dust(items, n_items));
         P.regular = all_regular(ctx, items, n_items);
         int grid = 1, variant = 3;
         launch_geometry(ctx, P, grid, variant);     // occupancy cached at soc_create
