@@ -58,8 +58,11 @@ __device__ __forceinline__ float u01(uint32_t x)
 __device__ __forceinline__ float one_minus_exp(float tau)
 {
     const float x = fmaxf(-tau, -87.0f);
-    const int k = __float2int_rn(__fmul_rn(x, 0x1.715476p+0f));         // rint(x / ln 2)
-    const float t = __int2float_rn(k);
+    // k = rint(x / ln 2): adding 1.5 2^23 rounds to the integer (ties to
+    // even, as rint) and leaves it in the low bits; two additions where the
+    // conversions to and from an integer run at a quarter of the rate
+    const float tk = __fadd_rn(__fmul_rn(x, 0x1.715476p+0f), 12582912.0f);
+    const float t = __fsub_rn(tk, 12582912.0f);
     float r = __fmaf_rn(-t, 0x1.62e4p-1f, x);                           // x - k ln2_hi
     r = __fmaf_rn(-t, 0x1.7f7d1cp-20f, r);                              //   - k ln2_lo
     float p = 0x1.a01a02p-13f;                                          // 1/7!
@@ -70,7 +73,7 @@ __device__ __forceinline__ float one_minus_exp(float tau)
     p = __fmaf_rn(p, r, 0.5f);
     p = __fmaf_rn(p, r, 1.0f);
     const float em1 = __fmul_rn(r, p);                                  // e^r - 1
-    const float sc = __uint_as_float((uint32_t)(k + 127) << 23);         // 2^k
+    const float sc = __uint_as_float((__float_as_uint(tk) << 23) + 0x3f800000u);   // 2^k
     const float q = __fmaf_rn(-sc, em1, __fsub_rn(1.0f, sc));
     return tau > 0.0f ? q : 0.0f;
 }
@@ -95,6 +98,8 @@ __device__ __forceinline__ float log_pos(float u)
     return __fadd_rn(__fadd_rn(__fmul_rn(t, 0x1.7f7d1cp-20f), lm), __fmul_rn(t, 0x1.62e4p-1f));
 }
 
-__device__ __forceinline__ float clamp01(float v) { return fminf(fmaxf(v, 0.0f), 1.0f); }
+// min(max(v, 0), 1) as the saturation of the operation that forms v (a NaN
+// gives 0, as max does); -0 becomes +0, which no later operation tells apart.
+__device__ __forceinline__ float clamp01(float v) { return __saturatef(v); }
 
 }  // namespace soc

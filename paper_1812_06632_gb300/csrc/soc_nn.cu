@@ -755,9 +755,9 @@ struct WgradArgs {
 //
 // Warps 0-15 copy (16-byte cp.async; out-of-volume voxels are written as
 // zeros), one thread of warp 16 issues the MMAs, and warps 0-3 read the sums
-// out at the end.  The copies' address arithmetic is what bounds the kernel
-// at 64^3, 16 -> 16: 80 us, 72 without the MMAs, 46 without the
-// copies.  A block takes the boxes [n_boxes b / chunks, n_boxes
+// out at the end.  The copies bound the kernel: at batch 4, 64^3,
+// 16 -> 16 it takes 80 us, 72 without the MMAs and 46 without the copies.
+// A block takes the boxes [n_boxes b / chunks, n_boxes
 // (b + 1) / chunks) and writes its sums to partial slice b;
 // reduce_partials_kernel adds the slices in order, so the result does not
 // depend on scheduling.  Rows of at most 8 voxels are taken in pairs (K = 16

