@@ -186,6 +186,14 @@ __device__ __forceinline__ void tmem_ld16(uint32_t addr, uint32_t (&rr)[16])
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+// zeros into 16 columns of the warp's 32 tensor-memory lanes (complete after
+// tcgen05.wait::st)
+__device__ __forceinline__ void tmem_zero16(uint32_t addr)
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1};"
+                 :: "r"(addr), "r"(0) : "memory");
+}
+
 // val[j] = 0 where mask[j] is not > 0 (8 values of a 16-byte aligned mask)
 __device__ __forceinline__ void apply_mask8(const bf16 *mask, float *val)
 {
@@ -293,7 +301,8 @@ struct ConvBlock {
 // Carve the bookkeeping after the stages, allocate tmem_cols columns of
 // tensor memory (warp 5) and initialise the barriers (thread 0).  Every
 // thread of the block calls it.
-__device__ __forceinline__ ConvBlock conv_block_begin(uint8_t *after_stages, int n_stages, uint32_t tmem_cols)
+__device__ __forceinline__ ConvBlock conv_block_begin(uint8_t *after_stages, int n_stages, uint32_t tmem_cols, int releasers = 1,
+                                                    int issuers = 1)
 {
     ConvBlock c;
     c.full = reinterpret_cast<uint64_t *>(after_stages);
@@ -312,13 +321,13 @@ __device__ __forceinline__ ConvBlock conv_block_begin(uint8_t *after_stages, int
     if (tid == 0) {
         for (int k = 0; k < n_stages; ++k) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&c.full[k])) : "memory");
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&c.empty[k])) : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(smem_u32(&c.empty[k])), "r"(releasers) : "memory");
         }
         for (int b = 0; b < 2; ++b) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&c.acc_full[b])) : "memory");
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 128;" :: "r"(smem_u32(&c.acc_empty[b])) : "memory");
         }
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(c.drain)) : "memory");
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(smem_u32(c.drain)), "r"(issuers) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         *c.s_fail = 0;
     }
@@ -343,7 +352,7 @@ __device__ __forceinline__ void conv_producer_tail(const ConvBlock &c, int n_sta
 // (the epilogue waited for the last box's accumulator, or, after a failure,
 // the MMA thread waits, bounded, for all it issued); a failure raises the
 // error flag.  Every thread calls it.
-__device__ __forceinline__ void conv_block_end(const ConvBlock &c, uint32_t tmem_cols)
+__device__ __forceinline__ void conv_block_end(const ConvBlock &c, uint32_t tmem_cols, int first_issuer = 5)
 {
     const int tid = threadIdx.x, warp = uniform_warp();
     __syncwarp();
@@ -351,7 +360,7 @@ __device__ __forceinline__ void conv_block_end(const ConvBlock &c, uint32_t tmem
     const bool ok = __syncthreads_and(!*reinterpret_cast<volatile int *>(c.s_fail));
     if (!ok) {
         if (tid == 0) atomicExch(&g_tc_error, 1);
-        if (warp == 5 && elect_one()) {
+        if (warp >= first_issuer && elect_one()) {
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
                          :: "r"(smem_u32(c.drain)) : "memory");
             mbar_wait(smem_u32(c.drain), 0);
@@ -695,6 +704,252 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv3d_slab_kernel(const __gr
         }
     }
     conv_block_end(cb, tmem_cols);
+}
+
+// ---------------------------------------------------------------------------
+// Plane-marching convolution.  An output box is G groups of 128 positions of
+// one sample's rows laid end to end with a pitch of W + 2 (the two voxels
+// past a row's end are computed and dropped), times Z planes.  For every
+// chunk of KC input channels each of the Z + 2 input planes arrives once, in
+// rows of W + 2 voxels (out-of-volume voxels read zero), and with that pitch
+// the A operand of tap (dy, dx) is the same 128 G rows of shared memory,
+// dy (W + 2) + dx rows on: no copy per x offset.  The three planes of outputs
+// that an input plane reaches lie side by side in tensor memory, so one MMA
+// of N = 3 n_tile columns serves three taps (dz = 2, 1, 0; fewer at the box's
+// ends).
+//
+// The slab kernel copies 36 KB a group of 128 voxels (64^3, 16 -> 16) and
+// issues 27 MMAs; here it is 10 KB and 9 (Z + 2) / Z MMAs.  At batch 4 that
+// layer takes 31.3 us against 52.6, 48 -> 16 72 against 133: 50 to 60 clocks an
+// MMA of 48 columns, which take the tensor core 44, the rest being the
+// first copies and the last box's way out.
+//
+// Sums are formed in the slab kernel's order (chunk, dx, dz, dy, channels), so
+// both give the same bits.  MMAs of overlapping columns but different shape
+// or start are not ordered by the hardware, so each step's MMAs wait for the
+// step before.  To keep the tensor core busy meanwhile, a group has three
+// issuing warps, one per dx, that march three planes behind one another, on
+// accumulators that do not overlap: a step is 9 MMAs (KC = 16) a group, and
+// passes, chunks and boxes follow each other without a gap.  One warp for
+// all groups took 64 us on 16 -> 16, one per group 38.  The accumulators
+// start from zeros that the epilogue warps write; they are drained plane by
+// plane, by 8 warps (4: 40 us).  Weights of all chunks stay in shared memory.
+// Block organisation, barriers and the bounded waits are otherwise those of
+// conv3d_tma_kernel; a stage is a plane.
+// ---------------------------------------------------------------------------
+struct MarchArgs {
+    int N, D, H, W, Cin, Cout;
+    int G, Z, n_rows, tiles_m, tiles_z;
+    ConvOut o;
+};
+
+constexpr int kMarchMaxGroups = 5, kMarchMaxChunks = 8, kMarchMaxZ = 16, kMarchEpi = 8;     // kMarchEpi: epilogue warps
+// w_full, done, and acc_full and acc_empty of two boxes
+constexpr int kMarchBars = kMarchMaxChunks + kMarchMaxGroups + 4 * kMarchMaxZ;
+
+template <int KC>
+__global__ void __launch_bounds__(32 * (kMarchEpi + 1 + 3 * kMarchMaxGroups), 1) conv3d_march_kernel(const __grid_constant__ CUtensorMap map_in,
+                                                                    const __grid_constant__ CUtensorMap map_w,
+                                                                    const MarchArgs a, int n_tile, uint32_t tmem_cols,
+                                                                    int n_slots, int plane_bytes)
+{
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    constexpr int kRow = KC * 2;
+    const int pitch = a.W + 2, planes = a.Z + 2;
+    const int n_chunks = a.Cin / KC;
+    const int tap_bytes = n_tile * kRow, w_bytes = 27 * tap_bytes;
+    const int w_off = n_slots * plane_bytes;
+    // weights landed per chunk, MMAs done per group, output planes of box i
+    // complete / drained at (i mod 2) kMarchMaxZ + z
+    uint64_t *const w_full = reinterpret_cast<uint64_t *>(smem + w_off + n_chunks * w_bytes);
+    uint64_t *const done = w_full + kMarchMaxChunks;
+    uint64_t *const acc_full = done + kMarchMaxGroups, *const acc_empty = acc_full + 2 * kMarchMaxZ;
+    const int tid = threadIdx.x, warp = uniform_warp();
+    if (tid == 0) {
+        for (int c = 0; c < n_chunks; ++c)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&w_full[c])) : "memory");
+        for (int q = 0; q < a.G; ++q)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 3;" :: "r"(smem_u32(&done[q])) : "memory");
+        for (int k = 0; k < 2 * kMarchMaxZ; ++k) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(smem_u32(&acc_full[k])), "r"(a.G) : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 128;" :: "r"(smem_u32(&acc_empty[k])) : "memory");
+        }
+    }
+    const ConvBlock cb = conv_block_begin(reinterpret_cast<uint8_t *>(w_full + kMarchBars), n_slots, tmem_cols, a.G, 3 * a.G);
+    uint64_t *const full = cb.full, *const empty = cb.empty;
+    int *const s_fail = cb.s_fail;
+    volatile int *fail = s_fail;
+    const uint32_t tmem = cb.tmem;
+    const uint32_t smem0 = smem_u32(smem);
+    const int n0 = blockIdx.y * n_tile;
+    const int n_boxes = a.tiles_m * a.tiles_z * a.N;
+
+    if (warp == kMarchEpi) {
+        if (elect_one()) {
+            asm volatile("prefetch.tensormap [%0];" :: "l"(reinterpret_cast<uint64_t>(&map_in)) : "memory");
+            asm volatile("prefetch.tensormap [%0];" :: "l"(reinterpret_cast<uint64_t>(&map_w)) : "memory");
+            const uint32_t tx_bytes = (uint32_t)(a.n_rows * pitch * kRow);
+            int st = 0, issued = 0, w_issued = 0;
+            uint32_t ph = 0;
+            bool stop = false;
+            for (int box = blockIdx.x; box < n_boxes && !stop && !*fail; box += gridDim.x) {
+                const int tm = box % a.tiles_m, q = box / a.tiles_m;
+                const int tz = q % a.tiles_z, nn = q / a.tiles_z;
+                const int y0 = tm * a.G * 128 / pitch - 1, z0 = tz * a.Z - 1;
+                for (int c = 0; c < n_chunks && !stop; ++c) {
+                    if (box == (int)blockIdx.x) {
+                        // weights of tap (dz, dy, dx) at block (3 dx + dy) 3 + 2 - dz
+                        const uint32_t bar = smem_u32(&w_full[c]);
+                        mbar_expect_tx(bar, (uint32_t)w_bytes);
+                        for (int t = 0; t < 27; ++t)
+                            tma_load_2d(smem0 + (uint32_t)(w_off + c * w_bytes + t * tap_bytes), &map_w,
+                                        (9 * (2 - t % 3) + 3 * (t / 3 % 3) + t / 9) * a.Cin + c * KC, n0, bar);
+                        ++w_issued;
+                    }
+                    for (int pl = 0; pl < planes; ++pl) {
+                        if (issued >= n_slots && !mbar_wait(smem_u32(&empty[st]), ph ^ 1u)) {
+                            atomicExch(s_fail, 1);
+                            stop = true;
+                            break;
+                        }
+                        if (*fail) { stop = true; break; }
+                        const uint32_t dst = smem0 + (uint32_t)(st * plane_bytes);
+                        const uint32_t bar = smem_u32(&full[st]);
+                        mbar_expect_tx(bar, tx_bytes);
+                        tma_load_5d(dst, &map_in, c * KC, -1, y0, z0 + pl, nn, bar);
+                        ++issued;
+                        if (++st == n_slots) { st = 0; ph ^= 1u; }
+                    }
+                }
+            }
+            conv_producer_tail(cb, n_slots, issued);
+            for (int c = 0; c < w_issued; ++c) mbar_wait(smem_u32(&w_full[c]), 0);
+        }
+    } else if (warp > kMarchEpi) {
+        if (elect_one()) {
+            const int q = (warp - kMarchEpi - 1) / 3, dx = (warp - kMarchEpi - 1) - 3 * q;
+            const uint32_t bar_done = smem_u32(&done[q]);
+            const uint64_t d0 = smem_desc_sw(0, kRow);
+            const uint32_t hi = (uint32_t)(d0 >> 32), lo0 = (uint32_t)d0 + (smem0 >> 4);
+            const uint32_t row16 = kRow >> 4, tap16 = (uint32_t)tap_bytes >> 4, plane16 = (uint32_t)plane_bytes >> 4;
+            const uint32_t dy16 = (uint32_t)pitch * row16;
+            const uint32_t idesc1 = mma_idesc(128, n_tile), idesc_n = mma_idesc(128, 2 * n_tile) - idesc1;
+            uint32_t round = 0;
+            bool ok = true;
+            // the group's three warps go step by step together: the MMAs of
+            // the step before have completed
+            auto begin_step = [&] {
+                if (round > 0 && !mbar_wait(bar_done, (round - 1u) & 1u)) ok = false;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            };
+            auto end_step = [&] {
+                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
+                             :: "r"(bar_done) : "memory");
+                ++round;
+            };
+            auto idle = [&](int n) {
+                for (int k = 0; k < n && ok; ++k) { begin_step(); end_step(); }
+            };
+            idle(3 * dx);
+            int s = 0, i = 0;
+            uint32_t ph = 0;
+            for (int box = blockIdx.x; box < n_boxes && ok; box += gridDim.x, ++i) {
+                const int b = i & 1;
+                const uint32_t off = (uint32_t)(box % a.tiles_m * a.G * 128 % pitch);
+                const uint32_t a_box = lo0 + (off + 128u * (uint32_t)q + (uint32_t)dx) * row16;
+                for (int c = 0; c < n_chunks && ok; ++c) {
+                    if (i == 0 && !mbar_wait(smem_u32(&w_full[c]), 0)) { ok = false; break; }
+                    const uint32_t b_dx = lo0 + ((uint32_t)(w_off + c * w_bytes) >> 4) + (uint32_t)(9 * dx) * tap16;
+                    uint32_t acc = tmem + (uint32_t)((b * a.G + q) * a.Z * n_tile);
+                    for (int pl = 0; pl < planes; ++pl) {
+                        if (!mbar_wait(smem_u32(&full[s]), ph) || *fail) { ok = false; break; }
+                        if (c == 0 && dx == 0 && pl < a.Z &&
+                            !mbar_wait(smem_u32(&acc_empty[b * kMarchMaxZ + pl]), (uint32_t)(i >> 1) & 1u)) {
+                            ok = false;
+                            break;
+                        }
+                        begin_step();
+                        if (!ok) break;
+                        // taps dz = min(pl, 2) down to max(0, pl - Z + 1), output planes max(0, pl - 2) up
+                        const uint32_t n_dz = (uint32_t)(min(pl, 2) - max(0, pl - a.Z + 1));
+                        const uint32_t idesc = idesc1 + n_dz * idesc_n;
+                        const uint32_t b0 = b_dx + (uint32_t)(2 - min(pl, 2)) * tap16;
+                        const uint32_t a0 = a_box + (uint32_t)s * plane16;
+#pragma unroll
+                        for (int dy = 0; dy < 3; ++dy)
+#pragma unroll
+                            for (int j = 0; j < KC / 16; ++j)
+                                mma_f16(acc, a0 + (uint32_t)dy * dy16 + 2u * j, hi, b0 + (uint32_t)dy * 3u * tap16 + 2u * j,
+                                        hi, idesc);
+                        end_step();
+                        if (dx == 2) {
+                            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
+                                         :: "r"(smem_u32(&empty[s])) : "memory");
+                            if (c + 1 == n_chunks && pl >= 2)
+                                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
+                                             :: "r"(smem_u32(&acc_full[b * kMarchMaxZ + pl - 2])) : "memory");
+                        }
+                        if (pl >= 2) acc += (uint32_t)n_tile;
+                        if (++s == n_slots) { s = 0; ph ^= 1u; }
+                    }
+                    // the next chunk's first pass follows the last one's
+                    // three planes behind (another box has other accumulators)
+                    if (c + 1 < n_chunks) idle(9 - planes);
+                }
+            }
+            idle(6 - 3 * dx);
+            if (ok && round > 0 && !mbar_wait(bar_done, (round - 1u) & 1u)) ok = false;
+            if (!ok) atomicExch(s_fail, 1);
+        }
+    } else {
+        // epilogue: warps 0-3 the even planes, 4-7 the odd ones; accumulator
+        // row r of group q = position m = 128 (tm G + q) + r of the plane.
+        // Zeros go back for the box after next.
+        const int half = warp >> 2, r = tid & 127;
+        const uint32_t lane0 = tmem + ((uint32_t)(r & 96) << 16);
+        const int buf_cols = a.G * a.Z * n_tile;
+        for (int c = 0; c < buf_cols; c += 16) tmem_zero16(lane0 + (uint32_t)(half * buf_cols + c));
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        for (int k = 0; k < kMarchMaxZ; ++k)
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_u32(&acc_empty[half * kMarchMaxZ + k])) : "memory");
+        int i = 0;
+        bool stop = false;
+        for (int box = blockIdx.x; box < n_boxes && !stop; box += gridDim.x, ++i) {
+            const int b = i & 1;
+            const int tm = box % a.tiles_m, qq = box / a.tiles_m;
+            const int tz = qq % a.tiles_z, nn = qq / a.tiles_z;
+            int row[kMarchMaxGroups];            // y W + x, or -1 outside
+#pragma unroll
+            for (int q = 0; q < kMarchMaxGroups; ++q) {
+                const int m = (tm * a.G + q) * 128 + r, y = m / pitch, x = m - y * pitch;
+                row[q] = x < a.W && y < a.H ? y * a.W + x : -1;
+            }
+            for (int zl = half; zl < a.Z; zl += 2) {
+                const bool ready = mbar_wait(smem_u32(&acc_full[b * kMarchMaxZ + zl]), (uint32_t)(i >> 1) & 1u);
+                if (__any_sync(0xffffffffu, !ready || *fail)) { atomicExch(s_fail, 1); stop = true; break; }
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const int z = tz * a.Z + zl;
+                const long long v0 = ((long long)nn * a.D + z) * a.H * a.W;
+#pragma unroll
+                for (int q = 0; q < kMarchMaxGroups; ++q) {
+                    if (q >= a.G) break;
+                    const uint32_t row_addr = lane0 + (uint32_t)(((b * a.G + q) * a.Z + zl) * n_tile);
+                    for (int c = 0; c < n_tile; c += 16) {
+                        uint32_t rr[16];
+                        tmem_ld16(row_addr + (uint32_t)c, rr);
+                        tmem_zero16(row_addr + (uint32_t)c);
+                        if (z < a.D && row[q] >= 0) store_row16(a.o, v0 + row[q], n0 + c, rr);
+                    }
+                }
+                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_u32(&acc_empty[b * kMarchMaxZ + zl])) : "memory");
+            }
+        }
+    }
+    conv_block_end(cb, tmem_cols, kMarchEpi + 1);
 }
 
 // Wt[ci][t][co] = W[co][26 - t][ci]: weights of the transposed convolution.
@@ -1653,6 +1908,136 @@ cudaError_t slab_launch(const ConvArgs &a, const SlabPlan &p, int sms, cudaStrea
     return cudaGetLastError();
 }
 
+// Plan of the plane-marching kernel for a shape with slab plan p (whose K
+// chunk it takes: the sums' order depends on it), or false where the slab
+// kernel is the faster one.  Boxes of G groups x Z planes and channel tiles
+// are scored by clocks: the MMAs (36 + 0.22 N each), a step's wait for its
+// own MMAs (400 and 60 an MMA of the group) and the copies at 20 bytes a clock,
+// times the rounds of boxes a block walks.  7 planes are alive between the
+// first pass and the last, and a single-chunk box takes 5 steps at least (its
+// accumulators are drained while the next box is computed).
+//
+// The line between the two kernels, measured at 16 shapes x 14 pairs of
+// channel counts: where the slab plan has less than 4 accumulators (grids
+// that hardly fill the SMs) the march is 0.73 to 1.0 times as fast, one chain
+// of dependent steps being all a block has; where all its weights fit only
+// beside a channel tile of half the slab's or less, every input is copied
+// twice as often or more: 0.53 to 1.35 (64^3 x 2, 128 -> 128: 434 us against
+// 753).  Elsewhere it is 1.06 to 2.45 times as fast (64^3 x 4: 16 -> 16 52.6
+// -> 31.3 us, 48 -> 16 133 -> 72, 16 -> 48 85 -> 66; 32^3 x 4: 32 -> 32 20.9 ->
+// 18.6, 32 -> 96 40 -> 29) but for 16^3 x 16, 64 -> 64 (31 against 36), where
+// the estimates lie as close as 1.11.
+struct MarchPlan {
+    int G, Z, n_tile, n_rows, n_slots, plane_bytes, bytes, tiles_m, tiles_z;
+    double clocks;
+};
+
+// Clocks of the slab kernel by the same estimates (its MMAs 1.3 times as long)
+double slab_clocks(const ConvArgs &a, const SlabPlan &p, int sms)
+{
+    const int grid_y = a.Cout / p.n_tile, n_chunks = a.Cin / p.kc;
+    const long long boxes = (long long)((a.H + p.by - 1) / p.by) * ((a.D + p.bz - 1) / p.bz) * a.N;
+    const long long grid_x = std::min<long long>(boxes, std::max(1, sms * p.per_sm / grid_y));
+    const double rounds = (double)((boxes + grid_x - 1) / grid_x);
+    const double per_sm = (double)std::min<long long>(p.per_sm, (grid_x * grid_y + sms - 1) / sms);
+    const double stage = (double)a.W * (p.by + 2) * (p.bz + 2) * p.kc * 2 + 9. * p.n_tile * p.kc * 2;
+    const double mma = 27. * n_chunks * (p.kc / 16) * p.n_acc * std::max(39., 36. + 0.22 * p.n_tile) * 1.3;
+    return rounds * per_sm * std::max(3. * n_chunks * stage / 20., mma);
+}
+
+bool march_plan(const ConvArgs &a, const SlabPlan &p, int sms, int sm_smem, int blk_max, MarchPlan &best)
+{
+    const int kc = p.kc;
+    if (p.n_acc < 4 || a.H > (1 << 20) || a.Cin / kc > kMarchMaxChunks) return false;
+    const int pitch = a.W + 2, n_chunks = a.Cin / kc, row = kc * 2;
+    const int groups = (a.H * pitch - 2 + 127) / 128;
+    const int fixed = 1024 + 8 * (2 * 32 + 5) + 8 + 8 * kMarchBars;
+    best.clocks = 0.;
+    for (int n_tile = 16; n_tile <= 80 && n_tile <= a.Cout; n_tile += 16) {
+        if (a.Cout % n_tile) continue;
+        const int w_bytes = 27 * n_tile * row * n_chunks;
+        if (w_bytes + fixed >= blk_max) break;
+        const int grid_y = a.Cout / n_tile;
+        for (int G = 1; G <= kMarchMaxGroups && G <= groups; ++G) {
+            const int n_rows = (128 * G + 3 * pitch + 1 + pitch - 1) / pitch;
+            if (n_rows > 256) break;
+            const int plane = (n_rows * pitch * row + 1023) / 1024 * 1024;
+            const int tiles_m = (groups + G - 1) / G;
+            for (int Z = 1; Z <= kMarchMaxZ && Z <= a.D && G * Z * n_tile <= 256; ++Z) {
+                const int slots = std::min(32, (blk_max - fixed - w_bytes) / plane);
+                const int steps = (n_chunks - 1) * std::max(9, Z + 2) + Z + 2;      // of a box
+                if (slots < 7) break;
+                if (steps < 5) continue;
+                const int tiles_z = (a.D + Z - 1) / Z;
+                const long long boxes = (long long)tiles_m * tiles_z * a.N;
+                const long long grid_x = std::min<long long>(boxes, std::max(1, sms / grid_y));
+                const double rounds = (double)((boxes + grid_x - 1) / grid_x);
+                const double mma = 9. * n_chunks * (Z + 2) * G * (kc / 16) * (36. + 0.22 * 3. * n_tile);
+                const double wait = steps * (400. + 3. * (kc / 16) * 60.);
+                const double feed = (double)n_chunks * (Z + 2) * plane / 20.;
+                const double t = rounds * std::max(std::max(mma, wait), feed) + 6. * wait / steps + w_bytes / 20.;
+                if (best.clocks == 0. || t < best.clocks)
+                    best = MarchPlan{G, Z, n_tile, n_rows, slots, plane, 0, tiles_m, tiles_z, t};
+            }
+        }
+    }
+    // 2000: a launch's own clocks, the same for both
+    if (best.clocks == 0. || 2 * best.n_tile <= p.n_tile || slab_clocks(a, p, sms) + 2000. < 1.2 * (best.clocks + 2000.))
+        return false;
+    best.bytes = 1024 + best.n_slots * best.plane_bytes + 27 * best.n_tile * row * n_chunks + 8 * (2 * best.n_slots + 5) + 8 +
+                 8 * kMarchBars;
+    // padded so that one block is resident on an SM
+    best.bytes = std::min(std::max(best.bytes, sm_smem / 2 + 1024), blk_max);
+    return true;
+}
+
+template <int KC>
+cudaError_t march_launch(const ConvArgs &a, const MarchPlan &p, int sms, cudaStream_t s)
+{
+    auto encode = encode_tiled();
+    if (!encode) return cudaErrorNotSupported;
+    const uintptr_t in_addr = reinterpret_cast<uintptr_t>(a.in + a.in_off);
+    if ((in_addr & 15u) || (reinterpret_cast<uintptr_t>(a.w) & 15u)) return cudaErrorInvalidValue;
+    MarchArgs t{};
+    t.N = a.N; t.D = a.D; t.H = a.H; t.W = a.W; t.Cin = a.Cin; t.Cout = a.Cout;
+    t.G = p.G; t.Z = p.Z; t.n_rows = p.n_rows; t.tiles_m = p.tiles_m; t.tiles_z = p.tiles_z;
+    t.o = conv_out(a);
+    constexpr CUtensorMapSwizzle sw = KC == 16 ? CU_TENSOR_MAP_SWIZZLE_32B : CU_TENSOR_MAP_SWIZZLE_64B;
+    CUtensorMap map_in, map_w;
+    {
+        const cuuint64_t dims[5] = {(cuuint64_t)a.Cin, (cuuint64_t)a.W, (cuuint64_t)a.H, (cuuint64_t)a.D,
+                                    (cuuint64_t)a.N};
+        const cuuint64_t vb = (cuuint64_t)a.in_stride * 2;
+        const cuuint64_t strides[4] = {vb, vb * a.W, vb * a.W * a.H, vb * a.W * a.H * a.D};
+        const cuuint32_t box[5] = {(cuuint32_t)KC, (cuuint32_t)a.W + 2, (cuuint32_t)p.n_rows, 1, 1};
+        const cuuint32_t es[5] = {1, 1, 1, 1, 1};
+        if (encode(&map_in, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, reinterpret_cast<void *>(in_addr), dims, strides, box,
+                   es, CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return cudaErrorInvalidValue;
+    }
+    {
+        const cuuint64_t dims[2] = {(cuuint64_t)27 * a.Cin, (cuuint64_t)a.Cout};
+        const cuuint64_t strides[1] = {(cuuint64_t)27 * a.Cin * 2};
+        const cuuint32_t box[2] = {(cuuint32_t)KC, (cuuint32_t)p.n_tile};
+        const cuuint32_t es[2] = {1, 1};
+        if (encode(&map_w, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<bf16 *>(a.w), dims, strides, box, es,
+                   CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return cudaErrorInvalidValue;
+    }
+    uint32_t cols = 32;
+    while ((int)cols < 2 * p.G * p.Z * p.n_tile) cols <<= 1;
+    const cudaError_t e = kernel_setup<conv3d_march_kernel<KC>, true>();
+    if (e != cudaSuccess) return e;
+    const int grid_y = a.Cout / p.n_tile;
+    const long long n_boxes = (long long)t.tiles_m * t.tiles_z * a.N;
+    dim3 grid((unsigned)std::min<long long>(n_boxes, std::max(1, sms / grid_y)), (unsigned)grid_y);
+    conv3d_march_kernel<KC><<<grid, 32 * (kMarchEpi + 1 + 3 * p.G), p.bytes, s>>>(map_in, map_w, t, p.n_tile, cols, p.n_slots,
+                                                              p.plane_bytes);
+    return cudaGetLastError();
+}
+
 // The slab-fed kernel where its plan applies, else the per-tap kernel with K
 // chunks of 64, 32 or 16 input channels (the largest dividing C_in).
 cudaError_t conv_launch(const ConvArgs &a, cudaStream_t s)
@@ -1660,6 +2045,9 @@ cudaError_t conv_launch(const ConvArgs &a, cudaStream_t s)
     const int sms = device_limits().sms, sm_smem = device_limits().sm_smem, blk_max = device_limits().blk_max;
     SlabPlan p{};
     if (slab_plan(a, sms, sm_smem, blk_max, p)) {
+        MarchPlan m{};
+        if (march_plan(a, p, sms, sm_smem, blk_max, m))
+            return p.kc == 32 ? march_launch<32>(a, m, sms, s) : march_launch<16>(a, m, sms, s);
         if (p.kc == 32)
             return p.n_acc == 4 ? slab_launch<32, 4>(a, p, sms, s)
                                 : (p.n_acc == 2 ? slab_launch<32, 2>(a, p, sms, s) : slab_launch<32, 1>(a, p, sms, s));

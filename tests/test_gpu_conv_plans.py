@@ -57,6 +57,17 @@ def test_conv_slabs(libsoc, shape, cin, cout):
     assert libsoc.nn_error_flag() == 0
 
 
+# the plane-marching kernel: boxes that end in the middle of a row, of a group
+# and of their planes, the narrowest and widest rows, fewer planes than a box
+# may have, one to four K chunks of 16 or 32, channel tiles of 16, 48 and 80
+@pytest.mark.parametrize("shape,cin,cout", [((2, 37, 40, 64), 16, 48), ((3, 50, 17, 16), 64, 32),
+                                             ((1, 39, 24, 128), 48, 16), ((60, 5, 21, 8), 16, 96),
+                                             ((4, 13, 70, 32), 32, 32), ((30, 3, 40, 32), 16, 16),
+                                             ((90, 7, 16, 8), 32, 80)])
+def test_conv_marches(libsoc, shape, cin, cout):
+    test_conv_slabs(libsoc, shape, cin, cout)
+
+
 @pytest.mark.parametrize("shape,cin,cout", [((1, 1, 1, 1), 16, 16), ((2, 3, 5, 8), 16, 32), ((1, 4, 7, 9), 32, 16),
                                              ((1, 3, 9, 16), 64, 48), ((1, 2, 11, 17), 128, 16), ((2, 2, 3, 65), 16, 80),
                                              ((1, 3, 2, 130), 48, 32), ((3, 6, 6, 4), 256, 64), ((1, 20, 21, 33), 16, 16),
