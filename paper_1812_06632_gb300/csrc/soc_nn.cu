@@ -1010,8 +1010,12 @@ struct WgradArgs {
 //
 // Warps 0-15 copy (16-byte cp.async; out-of-volume voxels are written as
 // zeros), one thread of warp 16 issues the MMAs, and warps 0-3 read the sums
-// out at the end.  The copies bound the kernel: at batch 4, 64^3,
-// 16 -> 16 it takes 80 us, 72 without the MMAs and 46 without the copies.
+// out at the end.  The copying warps' instructions bound the kernel (two a
+// clock and SM, half the issue slots, at 52 a copy when rows were brought one
+// plane and shift at a time: 80 us at batch 4, 64^3, 16 -> 16; 66 with all
+// planes or shifts of a piece together, 46 without the copies).  Not faster:
+// TMA boxes of 8 channels (92 us: 16-byte rows at 8 bytes a clock) and two of
+// the three x planes moved within shared memory (91 us).
 // A block takes the boxes [n_boxes b / chunks, n_boxes
 // (b + 1) / chunks) and writes its sums to partial slice b;
 // reduce_partials_kernel adds the slices in order, so the result does not
@@ -1081,12 +1085,16 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv3d_wgrad_tc_kernel(const Wg
     float bias_sum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 
     if (warp < kWgCopyWarps) {
-        // lane's first piece of a row of x and of gy (channel groups fastest),
-        // and what 32 pieces further on means in global and shared memory
+        // A unit is 32 pieces of a row (channel groups fastest), brought for
+        // all three planes (x) or shifts (gy) at once, so that a piece costs
+        // few instructions beyond its copy.  Unit u of x is k = u mod x_per of
+        // row u / x_per; warps take every 16th unit, by carries.
         const int ax = lane / HN, ah = lane % HN;
-        const uint32_t a_dst = (uint32_t)(ah * 3 * a.wp + ax) * 16u;
-        const int a_src = ax * a.x_stride + ah * 8, a_step = (32 / HN) * a.x_stride;
-        const int q0 = lane / nn, r0 = lane - q0 * nn, dq = 32 / nn, dr = 32 - dq * nn;
+        const int x_per = (a.bxk + 32 / HN - 1) / (32 / HN), gy_per = (a.bxk * nn + 31) / 32;
+        const int xy0 = warp / x_per, xk0 = warp - xy0 * x_per, xdy = kWgCopyWarps / x_per, xdk = kWgCopyWarps - xdy * x_per;
+        const int gy0 = warp / gy_per, gk0 = warp - gy0 * gy_per, gdy = kWgCopyWarps / gy_per, gdk = kWgCopyWarps - gdy * gy_per;
+        const uint32_t inv_nn = 65536u / (uint32_t)nn + 1u;      // i / nn = (i inv_nn) >> 16 for the i < 64 nn <= 640 met here
+        const uint32_t wp16 = (uint32_t)a.wp * 16u, bp16 = (uint32_t)a.bp * 16u;
         int st = 0, issued = 0, told = 0;
         int turn = (box0 + n_ci - ci_tile) % n_ci;         // 0: this block sums the next box's gy
         uint32_t ph = 0;
@@ -1137,38 +1145,36 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv3d_wgrad_tc_kernel(const Wg
             const uint32_t A0 = smem0 + (uint32_t)(st * a.stage_bytes), B0 = A0 + (uint32_t)a.a_bytes;
             const long long row0 = nzy * a.H + y0;
             const bf16 *const xb = a.x + row0 * x_row + (long long)x0 * a.x_stride + a.x_off + ci0;
-            const bf16 *const gb = a.gy + row0 * gy_row + a.gy_off + co0;
+            const bf16 *const gb = a.gy + row0 * gy_row + (long long)x0 * a.gy_stride + a.gy_off + co0;
             const int wx = a.W - x0;                       // voxels of the rows left from x0 on
-            for (int r = warp; r < 3 * (a.by + 2); r += kWgCopyWarps) {
-                const int yp = r / 3, zp = r - 3 * yp;
-                const bool row = (unsigned)(y0 + yp - 1) < (unsigned)a.H && (unsigned)(z + zp - 1) < (unsigned)a.D;
-                const bf16 *const base = row ? xb + ((zp - 1) * x_plane + (yp - 1) * x_row) : a.x;
-                const int lim = row ? wx : 0;
-                uint32_t dst = A0 + (uint32_t)((yp * HN * 3 + zp) * a.wp) * 16u + a_dst;
-                int off = a_src;
-#pragma unroll 4
-                for (int xq = ax; xq < a.bxk; xq += 32 / HN) {
-                    const bool in = xq < lim;
-                    cp_async16(dst, base + (in ? off : 0), in ? 16u : 0u);
-                    dst += 32 / HN * 16;
-                    off += a_step;
+            const bool below = z > 0, above = z + 1 < a.D;
+            for (int yp = xy0, k = xk0; yp < a.by + 2;) {
+                const int xq = k * (32 / HN) + ax;
+                const bool in = (unsigned)(y0 + yp - 1) < (unsigned)a.H && xq < wx;
+                const bf16 *const src = xb + ((yp - 1) * x_row + xq * a.x_stride + ah * 8);
+                const uint32_t dst = A0 + (uint32_t)((yp * HN + ah) * 3) * wp16 + (uint32_t)xq * 16u;
+                if (xq < a.bxk) {
+                    cp_async16(dst, in && below ? src - x_plane : a.x, in && below ? 16u : 0u);
+                    cp_async16(dst + wp16, in ? src : a.x, in ? 16u : 0u);
+                    cp_async16(dst + 2u * wp16, in && above ? src + x_plane : a.x, in && above ? 16u : 0u);
                 }
+                yp += xdy; k += xdk;
+                if (k >= x_per) { k -= x_per; ++yp; }
             }
-            for (int r = warp; r < 3 * a.by; r += kWgCopyWarps) {
-                const int y = r / 3, c = r - 3 * y;
-                const bool row = y0 + y < a.H;
-                // shared voxel q is voxel x0 + q - (c - 1) of the row
-                const bf16 *const base = row ? gb + y * gy_row : a.gy;
-                const int sh = x0 - (c - 1), len = row ? a.W : 0;
-                const uint32_t dst = B0 + (uint32_t)(r * nn * a.bp) * 16u;
-#pragma unroll 4
-                for (int xq = q0, g = r0; xq < a.bxk;) {
-                    const bool in = (unsigned)(xq + sh) < (unsigned)len;
-                    cp_async16(dst + (uint32_t)(g * a.bp + xq) * 16u, base + (in ? (xq + sh) * a.gy_stride + g * 8 : 0),
-                               in ? 16u : 0u);
-                    xq += dq; g += dr;
-                    if (g >= nn) { g -= nn; ++xq; }
+            for (int y = gy0, k = gk0; y < a.by;) {
+                const int q = k * 32 + lane, xq = (int)((uint32_t)q * inv_nn >> 16), g = q - xq * nn;
+                // shared voxel xq of shift c is voxel x0 + xq - (c - 1) of the row
+                const int lim = y0 + y < a.H ? wx : -1;              // (wx >= 1)
+                const bf16 *const src = gb + (y * gy_row + xq * a.gy_stride + g * 8);
+                const uint32_t dst = B0 + (uint32_t)(3 * y * nn + g) * bp16 + (uint32_t)xq * 16u;
+                const bool p0 = xq + 1 < lim, p1 = xq < lim, p2 = xq <= lim && xq + x0 > 0;
+                if (xq < a.bxk) {
+                    cp_async16(dst, p0 ? src + a.gy_stride : a.gy, p0 ? 16u : 0u);
+                    cp_async16(dst + (uint32_t)nn * bp16, p1 ? src : a.gy, p1 ? 16u : 0u);
+                    cp_async16(dst + 2u * (uint32_t)nn * bp16, p2 ? src - a.gy_stride : a.gy, p2 ? 16u : 0u);
                 }
+                y += gdy; k += gdk;
+                if (k >= gy_per) { k -= gy_per; ++y; }
             }
             if (++seg == a.segs) {
                 seg = 0;
