@@ -414,7 +414,8 @@ soc_status soc_update_temperature_ali(soc_ctx *ctx, int cloud_id, const double *
  * enters from behind attenuated by the total optical depth.
  *   d_T     device float [n_cells];  d_map  device float [npy][npx].
  * FP32 cell-local traversal and segment optical depths as in the tracer;
- * the source function per cell and the accumulation along the ray in FP64.
+ * the source function per cell and the accumulation along the ray in pairs
+ * of FP32 numbers (high and low part, relative error about 2^-40).
  * Uses a per-context scratch of n_cells doubles (calls on one context must
  * not overlap on the GPU).  Asynchronous.
  * ------------------------------------------------------------------------ */

@@ -8,6 +8,9 @@
 // adjacent threads reading adjacent cells).  Sums and products are written
 // with the _rn intrinsics in a fixed order so that the absorbed power equals
 // a plain sequential FP64 evaluation bit for bit.
+// The dust weights, a Planck function per (leaf, frequency), are formed from
+// pairs of FP32 numbers and in FP64 only where their rounding needs it (the
+// FP64 pipe does 2 lanes a clock and SM).
 #include <cuda_runtime.h>
 #include <cstdint>
 #include <algorithm>
