@@ -142,8 +142,8 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, uint32
 // coordinates outside the volume read zeros, which is the convolution's
 // padding -- and a second one the weights (n_tile rows x KC), both with
 // rows of KC * 2 bytes in the hardware's 32/64/128-byte swizzle, which the
-// MMA's shared-memory descriptors name.  One thread issues the loads
-// (mbarrier with the expected byte count per stage), another the MMAs
+// MMA's shared-memory descriptors name.  Up to four threads issue the loads
+// (mbarrier with the expected byte count per stage), another one the MMAs
 // (committed to the stage's "empty" mbarrier), n_stages stages deep; every
 // wait is bounded (on a timeout the block raises the error flag, waits for
 // its loads and MMAs in flight, frees its tensor memory and returns).
@@ -338,13 +338,16 @@ __device__ __forceinline__ ConvBlock conv_block_begin(uint8_t *after_stages, int
     return c;
 }
 
-// The producer's last stages (issued: its copies so far, into stages
-// h mod n_stages): after a failure the copies in flight land, else the MMAs'
-// releases of them arrive, before the block leaves.  Bounded waits.
-__device__ __forceinline__ void conv_producer_tail(const ConvBlock &c, int n_stages, int issued)
+// A producer's last stages (its copies are those of steps first, first + by,
+// ... below issued, into stages h mod n_stages): after a failure the copies in
+// flight land, else the MMAs' releases of them arrive, before the block
+// leaves.  Bounded waits.
+__device__ __forceinline__ void conv_producer_tail(const ConvBlock &c, int n_stages, int issued, int first = 0, int by = 1)
 {
     const bool failed = *reinterpret_cast<volatile int *>(c.s_fail);
-    for (int h = (issued > n_stages ? issued - n_stages : 0); h < issued; ++h)
+    int h = first;
+    if (issued > n_stages && h < issued - n_stages) h += (issued - n_stages - h + by - 1) / by * by;
+    for (; h < issued; h += by)
         mbar_wait(smem_u32(failed ? &c.full[h % n_stages] : &c.empty[h % n_stages]), (uint32_t)(h / n_stages) & 1u);
 }
 
@@ -352,7 +355,7 @@ __device__ __forceinline__ void conv_producer_tail(const ConvBlock &c, int n_sta
 // (the epilogue waited for the last box's accumulator, or, after a failure,
 // the MMA thread waits, bounded, for all it issued); a failure raises the
 // error flag.  Every thread calls it.
-__device__ __forceinline__ void conv_block_end(const ConvBlock &c, uint32_t tmem_cols, int first_issuer = 5)
+__device__ __forceinline__ void conv_block_end(const ConvBlock &c, uint32_t tmem_cols, int first_issuer = 5, int issuers = 1)
 {
     const int tid = threadIdx.x, warp = uniform_warp();
     __syncwarp();
@@ -360,7 +363,7 @@ __device__ __forceinline__ void conv_block_end(const ConvBlock &c, uint32_t tmem
     const bool ok = __syncthreads_and(!*reinterpret_cast<volatile int *>(c.s_fail));
     if (!ok) {
         if (tid == 0) atomicExch(&g_tc_error, 1);
-        if (warp >= first_issuer && elect_one()) {
+        if (warp >= first_issuer && warp < first_issuer + issuers && elect_one()) {
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
                          :: "r"(smem_u32(c.drain)) : "memory");
             mbar_wait(smem_u32(c.drain), 0);
@@ -373,18 +376,21 @@ __device__ __forceinline__ void conv_block_end(const ConvBlock &c, uint32_t tmem
     }
 }
 
-// Persistent and warp-specialised: a block of 6 warps walks the output
-// boxes blockIdx.x, blockIdx.x + gridDim.x, ...  Warp 4 (lane 0) issues the
-// TMA loads into n_stages shared-memory stages, warp 5 (lane 0) the MMAs into
+// Persistent and warp-specialised: a block walks the output boxes blockIdx.x,
+// blockIdx.x + gridDim.x, ...  Warp 4 (and the warps after 5: one lane each)
+// issues the TMA loads into n_stages shared-memory stages, warp 5 the MMAs into
 // one of two accumulators in tensor memory (2 x n_tile columns), and warps
 // 0-3 (tensor-memory lanes 32w .. 32w + 31) drain the other accumulator:
 // loads of the next box, MMAs and the epilogue of the previous one overlap.
 // Barriers: full/empty per stage (TMA bytes arrived / MMAs done with it),
 // acc_full/acc_empty per accumulator (MMAs of a box done / epilogue done).
 constexpr int kConvThreads = 192;
+// producer warps of conv3d_tma_kernel, at most
+constexpr int kConvProducers = 4;
+constexpr int kTmaThreads = 32 * (5 + kConvProducers);
 
 template <int KC>
-__global__ void __launch_bounds__(kConvThreads) conv3d_tma_kernel(const __grid_constant__ CUtensorMap map_in,
+__global__ void __launch_bounds__(kTmaThreads) conv3d_tma_kernel(const __grid_constant__ CUtensorMap map_in,
                                                                   const __grid_constant__ CUtensorMap map_w,
                                                                   const TmaConvArgs a, int n_tile, uint32_t tmem_cols,
                                                                   int n_stages)
@@ -411,51 +417,63 @@ __global__ void __launch_bounds__(kConvThreads) conv3d_tma_kernel(const __grid_c
     const uint32_t tx_bytes = (uint32_t)(a.bx * a.by * a.bz * a.bn) * kRow + (uint32_t)b_bytes;
 
 
-    if (warp == 4) {
+    if (warp == 4 || warp > 5) {
+        // producers: the block's step g = (box, tap, chunk) goes into stage g
+        // mod n_stages, in round floor(g / n_stages), once the MMAs of step g -
+        // n_stages have released it.  One thread took about 560 clocks a
+        // step (8^3, 128 -> 128: 21 us, 17.5 here; a ragged 48 -> 32 layer 29,
+        // 21; 8 producers were slower than 4), so each of n_prod brings every
+        // n_prod-th step.  n_stages is a multiple of n_prod: a stage has one
+        // producer, which cannot be more than one round ahead of the phase
+        // that its wait's parity names.
+        const int n_prod = min(kConvProducers, n_stages);
         if (elect_one()) {
-            asm volatile("prefetch.tensormap [%0];" :: "l"(reinterpret_cast<uint64_t>(&map_in)) : "memory");
-            asm volatile("prefetch.tensormap [%0];" :: "l"(reinterpret_cast<uint64_t>(&map_w)) : "memory");
-            // producer: step g = (box, tap, chunk) into stage st = g mod
-            // n_stages, in round ph = floor(g / n_stages) mod 2, once the MMAs
-            // of step g - n_stages have released it
-            int st = 0, issued = 0;
+            const int p = warp == 4 ? 0 : warp - 5;
+            if (p == 0) {
+                asm volatile("prefetch.tensormap [%0];" :: "l"(reinterpret_cast<uint64_t>(&map_in)) : "memory");
+                asm volatile("prefetch.tensormap [%0];" :: "l"(reinterpret_cast<uint64_t>(&map_w)) : "memory");
+            }
+            int g = p, st = p, left = p, issued = 0;       // left: steps to go to the next one of this producer
             uint32_t ph = 0;
-            for (int box = blockIdx.x; box < n_boxes && !*fail; box += gridDim.x) {
+            bool stop = p >= n_prod;
+            for (int box = blockIdx.x; box < n_boxes && !stop && !*fail; box += gridDim.x) {
                 int q = box;
                 const int tx = q % a.tiles_x; q /= a.tiles_x;
                 const int ty = q % a.tiles_y; q /= a.tiles_y;
                 const int tz = q % a.tiles_z;
                 const int tn = q / a.tiles_z;
                 const int x0 = tx * a.bx - 1, y0 = ty * a.by - 1, z0 = tz * a.bz - 1, nb0 = tn * a.bn;
-                bool stop = false;
-                for (int tap = 0, dx = 0, dy = 0, dz = 0; tap < 27 && !stop; ++tap) {
-                    for (int c0 = 0; c0 < a.Cin; c0 += KC) {
-                        if (issued >= n_stages && !mbar_wait(smem_u32(&empty[st]), ph ^ 1u)) {
-                            atomicExch(s_fail, 1);
-                            stop = true;
-                            break;
-                        }
-                        if (*fail) { stop = true; break; }
-                        const uint32_t dst = smem0 + (uint32_t)(st * stage_bytes);
-                        const uint32_t bar = smem_u32(&full[st]);
-                        mbar_expect_tx(bar, tx_bytes);
-                        tma_load_5d(dst, &map_in, c0, x0 + dx, y0 + dy, z0 + dz, nb0, bar);
-                        tma_load_2d(dst + (uint32_t)a_bytes, &map_w, tap * a.Cin + c0, n0, bar);
-                        ++issued;
-                        if (++st == n_stages) { st = 0; ph ^= 1u; }
+                int t = left;
+                for (; t < steps; t += n_prod, g += n_prod) {
+                    const int tap = t / n_chunks, c0 = (t - tap * n_chunks) * KC;
+                    if (g >= n_stages && !mbar_wait(smem_u32(&empty[st]), ph ^ 1u)) {
+                        atomicExch(s_fail, 1);
+                        stop = true;
+                        break;
                     }
-                    // tap = 9 dz + 3 dy + dx
-                    if (++dx == 3) { dx = 0; if (++dy == 3) { dy = 0; ++dz; } }
+                    if (*fail) { stop = true; break; }
+                    const uint32_t dst = smem0 + (uint32_t)(st * stage_bytes);
+                    const uint32_t bar = smem_u32(&full[st]);
+                    mbar_expect_tx(bar, tx_bytes);
+                    tma_load_5d(dst, &map_in, c0, x0 + tap % 3, y0 + tap / 3 % 3, z0 + tap / 9, nb0, bar);
+                    tma_load_2d(dst + (uint32_t)a_bytes, &map_w, tap * a.Cin + c0, n0, bar);
+                    issued = g + 1;
+                    st += n_prod;
+                    if (st >= n_stages) { st -= n_stages; ph ^= 1u; }
                 }
-                if (stop) break;
+                left = t - steps;
             }
-            conv_producer_tail(cb, n_stages, issued);
+            conv_producer_tail(cb, n_stages, issued, p, n_prod);
         }
     } else if (warp == 5) {
         if (elect_one()) {
             // MMA issuer: box i into accumulator i % 2, once the epilogue has
             // drained box i - 2 from it
             const uint32_t idesc = mma_idesc(128, n_tile);
+            const uint64_t d0 = smem_desc_sw(0, kRow);
+            const uint32_t hi = (uint32_t)(d0 >> 32), lo0 = (uint32_t)d0 + (smem0 >> 4);
+            const uint32_t stage16 = (uint32_t)stage_bytes >> 4, a16 = (uint32_t)a_bytes >> 4;
+            uint32_t a0 = lo0;
             int st = 0, i = 0;
             uint32_t ph = 0;
             for (int box = blockIdx.x; box < n_boxes && !*fail; box += gridDim.x, ++i) {
@@ -473,19 +491,15 @@ __global__ void __launch_bounds__(kConvThreads) conv3d_tma_kernel(const __grid_c
                     }
                     if (*fail) break;
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const uint32_t a0 = smem0 + (uint32_t)(st * stage_bytes), b0 = a0 + (uint32_t)a_bytes;
 #pragma unroll
                     for (int j = 0; j < KC / 16; ++j) {
-                        const uint64_t ad = smem_desc_sw(a0 + j * 32, kRow);
-                        const uint64_t bd = smem_desc_sw(b0 + j * 32, kRow);
-                        const uint32_t acc = (t > 0 || j > 0) ? 1u : 0u;
-                        asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                                     " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-                                     :: "r"(acc_addr), "l"(ad), "l"(bd), "r"(idesc), "r"(acc) : "memory");
+                        if (j == 0) mma_f16<true>(acc_addr, a0, hi, a0 + a16, hi, idesc, t > 0 ? 1u : 0u);
+                        else mma_f16(acc_addr, a0 + 2u * j, hi, a0 + a16 + 2u * j, hi, idesc);
                     }
                     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
                                  :: "r"(smem_u32(&empty[st])) : "memory");
-                    if (++st == n_stages) { st = 0; ph ^= 1u; }
+                    a0 += stage16;
+                    if (++st == n_stages) { st = 0; ph ^= 1u; a0 = lo0; }
                 }
                 // the box's accumulator is complete once its MMAs are
                 asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
@@ -949,7 +963,7 @@ __global__ void __launch_bounds__(32 * (kMarchEpi + 1 + 3 * kMarchMaxGroups), 1)
             }
         }
     }
-    conv_block_end(cb, tmem_cols, kMarchEpi + 1);
+    conv_block_end(cb, tmem_cols, kMarchEpi + 1, 3 * a.G);
 }
 
 // Wt[ci][t][co] = W[co][26 - t][ci]: weights of the transposed convolution.
@@ -1772,12 +1786,13 @@ cudaError_t tma_launch(const ConvArgs &a, cudaStream_t s)
     // stages, 2 to 24 (a step is a fraction of a TMA round trip, so few blocks
     // want many: the 8^3 layers, 128 blocks, ran 2 stages each)
     const long long blocks = tiles * (a.Cout / n_tile);
-    const int per_sm = (int)std::min<long long>(std::min(8, std::min(512 / (int)cols, 2048 / kConvThreads)),
+    const int per_sm = (int)std::min<long long>(std::min(8, std::min(512 / (int)cols, 2048 / kTmaThreads)),
                                                 (blocks + sms - 1) / sms);
     const int stage_bytes = (128 + n_tile) * KC * 2;
     const int fixed = 1024 + 8 * (2 * 24 + 5) + 8;    // alignment, barriers, slot and flag
     int stages = (std::min(sm_smem / per_sm - 1024, blk_max) - fixed) / stage_bytes;
     stages = stages < 2 ? 2 : (stages > 24 ? 24 : stages);
+    stages -= stages % std::min(kConvProducers, stages);         // a stage has one producer
     const int need = 1024 + stages * stage_bytes + 8 * (2 * stages + 5) + 8;
     if (need > blk_max) return cudaErrorInvalidValue;
     // padded so that no more than per_sm blocks are resident on an SM
@@ -1791,13 +1806,13 @@ cudaError_t tma_launch(const ConvArgs &a, cudaStream_t s)
     const cudaError_t e = kernel_setup<conv3d_tma_kernel<KC>, true>(&regs);
     if (e != cudaSuccess) return e;
     const int warp_regs = ((regs + 7) / 8) * 8 * 32;
-    const int reg_blocks = 65536 / (warp_regs * (kConvThreads / 32));
+    const int reg_blocks = 65536 / (warp_regs * (kTmaThreads / 32));
     const int occ = std::max(1, std::min(per_sm, reg_blocks));
     const int grid_y = a.Cout / n_tile;
     // persistent: each block walks boxes gridDim.x apart
     const long long slots = std::max(1LL, (long long)sms * occ / grid_y);
     dim3 grid((unsigned)std::min(tiles, slots), (unsigned)grid_y);
-    conv3d_tma_kernel<KC><<<grid, kConvThreads, bytes, s>>>(map_in, map_w, t, n_tile, cols, stages);
+    conv3d_tma_kernel<KC><<<grid, kTmaThreads, bytes, s>>>(map_in, map_w, t, n_tile, cols, stages);
     return cudaGetLastError();
 }
 

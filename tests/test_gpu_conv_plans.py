@@ -68,6 +68,15 @@ def test_conv_marches(libsoc, shape, cin, cout):
     test_conv_slabs(libsoc, shape, cin, cout)
 
 
+# the per-tap kernel: two, three, four and many stages (as many producers, at
+# most four), several boxes a block, one and several K chunks
+@pytest.mark.parametrize("shape,cin,cout", [((2, 24, 24, 24), 64, 64), ((2, 24, 24, 24), 64, 128),
+                                             ((1, 20, 12, 24), 64, 256), ((2, 13, 10, 27), 48, 32),
+                                             ((3, 50, 21, 24), 16, 16), ((1, 2, 3, 5), 32, 16)])
+def test_conv_taps(libsoc, shape, cin, cout):
+    test_conv_slabs(libsoc, shape, cin, cout)
+
+
 @pytest.mark.parametrize("shape,cin,cout", [((1, 1, 1, 1), 16, 16), ((2, 3, 5, 8), 16, 32), ((1, 4, 7, 9), 32, 16),
                                              ((1, 3, 9, 16), 64, 48), ((1, 2, 11, 17), 128, 16), ((2, 2, 3, 65), 16, 80),
                                              ((1, 3, 2, 130), 48, 32), ((3, 6, 6, 4), 256, 64), ((1, 20, 21, 33), 16, 16),
